@@ -122,11 +122,12 @@ int claw_set_level(claw_ctx* ctx, int32_t level, const claw_box* boxes, int32_t 
 
 /* Chooses the tiling of the fused level-step for a level: tx x ty interior cells per tile,
  * the staging of the tile's q planes into shared memory (0 = cooperative loads,
- * 1 = tensor-memory-accelerator bulk copies into two buffers, 2 = bulk copies into one buffer with
- * three CTAs per SM, acoustics 32x16 with 256 threads only; 1 and 2 only when every box has even
- * nx and offsets) and
+ * 1 = tensor-memory-accelerator bulk copies into two buffers, 2 = bulk copies into one buffer,
+ * acoustics 32x16 with 256 threads and, in a uniform medium, 32x32 with 256; 1 and 2 only when every
+ * box has even nx and offsets) and
  * the threads per CTA (0 = default).  Supported for acoustics: 32x32 with 256 or 512 threads,
- * 32x16 with 256, 16x16 with 128; claw_set_level installs 32x32, 256 threads.  Supported for
+ * 32x16 with 256, 16x16 with 128, and in a uniform medium 32x16 with 352 and 16x16 with 192 too;
+ * claw_set_level installs 32x32, 256 threads.  Supported for
  * shallow water: 16x16 with 256 threads, 32x16 with 512; claw_set_level installs 16x16.  Once
  * chosen here, a level's tiling stays through later claw_set_level calls (with staging 0 when
  * the new boxes do not allow bulk copies), as does its claw_set_tile_walk choice.
@@ -141,11 +142,10 @@ int claw_set_tiling(claw_ctx* ctx, int32_t level, int32_t tx, int32_t ty, int32_
  * strides over the tiles, largest first.  walk = 1 (acoustics in a uniform medium, shallow water): the
  * tiles form columns, each box's tile columns continued into the same-level box directly above
  * when it has the same run, ilo and nx; every CTA takes one contiguous stretch of about equal
- * cost, and a tile that follows the tile below it in its CTA's stretch takes the edge values of
- * the rows they share from that tile instead of recomputing them.  Both give the same q_new, dt
- * and smax bit for bit.  walk = -1 (claw_set_level installs it): 1 for uniform-medium levels
- * with at least 8 tiles per SM, else 0 (shallow water measured faster striding).  A cell-wise
- * medium accepts 0 and -1 (which means 0).  A
+ * cost, and (shallow water) a tile that follows the tile below it in its CTA's stretch takes the
+ * edge values of the rows they share from that tile instead of recomputing them.  Both give the
+ * same q_new, dt and smax bit for bit.  walk = -1 (claw_set_level installs it): 0, which measured
+ * faster for either system.  A cell-wise medium accepts 0 and -1.  A
  * change rewrites the level's tile lists like claw_set_tiling.
  * Errors: CLAW_EINVAL, CLAW_ENOMEM, CLAW_ECUDA. */
 int claw_set_tile_walk(claw_ctx* ctx, int32_t level, int32_t walk);

@@ -26,8 +26,7 @@ StepArgs make_args(claw_ctx* ctx, int L, const double* q_old, double* q_new, con
     a.err = ctx->err;
     a.order = ctx->order;
     a.transverse = ctx->transverse;
-    a.rho0 = ctx->rho0;
-    a.K0 = ctx->K0;
+    a.set_medium(ctx->rho0, ctx->K0);
     a.grav = ctx->grav;
     a.swe = ctx->kind() == KIND_SWE;
     a.wait_polls = ctx->wait_polls;
@@ -315,11 +314,14 @@ int claw_set_tiling(claw_ctx* ctx, int32_t L, int32_t tx, int32_t ty, int32_t st
         ctx->kind() == KIND_SWE
             ? (tx == 16 && ty == 16 && (threads == 0 || threads == 256)) ||
                   (tx == 32 && ty == 16 && (threads == 0 || threads == 512))
-            : (tx == 32 && ty == 32 && (threads == 0 || threads == 256 || threads == 512)) ||
+            : (ctx->kind() == KIND_UNIFORM &&
+               ((tx == 32 && ty == 16 && threads == 352) || (tx == 16 && ty == 16 && threads == 192))) ||
+                  (tx == 32 && ty == 32 && (threads == 0 || threads == 256 || threads == 512)) ||
                   (tx == 32 && ty == 16 && (threads == 0 || threads == 256)) ||
                   (tx == 16 && ty == 16 && (threads == 0 || threads == 128));
     // staging 2 (one bulk-copy buffer, three CTAs per SM) exists for the acoustics 32x16 tiles
-    const bool staging2_ok = ctx->kind() != KIND_SWE && tx == 32 && ty == 16 && (threads == 0 || threads == 256);
+    const bool staging2_ok = (ctx->kind() != KIND_SWE && tx == 32 && ty == 16 && (threads == 0 || threads == 256)) ||
+                             (ctx->kind() == KIND_UNIFORM && tx == 32 && ty == 32 && (threads == 0 || threads == 256));
     if (!shape_ok || staging < 0 || staging > 2 || (staging == 2 && !staging2_ok) ||
         (staging >= 1 && !ctx->tma_ok[L]))
         return CLAW_EINVAL;

@@ -5,6 +5,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <cmath>
+
 #include <vector>
 
 #include "../../include/claw.h"
@@ -241,6 +243,15 @@ struct StepArgs {
     // scheme
     int order = 2, transverse = 2;
     double rho0 = 1.0, K0 = 1.0;   // uniform medium
+    double Z0 = 1.0, c0 = 1.0, iZ = 1.0;   // its impedance, speed and 1 / Z0 (set_medium)
+    void set_medium(double rho, double K)
+    {
+        rho0 = rho;
+        K0 = K;
+        Z0 = std::sqrt(K * rho);
+        c0 = std::sqrt(K / rho);
+        iZ = 1.0 / Z0;
+    }
     double grav = 0.0;             // shallow water
     int swe = 0;                   // 1: the shallow water system (the conservation fix reads it)
     const longlong2* ring = nullptr;   // not null: same-level and boundary ghosts are pulled from sources

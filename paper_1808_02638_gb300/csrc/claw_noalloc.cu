@@ -125,8 +125,7 @@ extern "C" int claw_level_step_noalloc(int32_t nx, int32_t ny, double dx, double
     a.err = reinterpret_cast<int*>(s);
     a.order = order;
     a.transverse = transverse;
-    a.rho0 = rho0;
-    a.K0 = K0;
+    a.set_medium(rho0, K0);
     const int grid = std::min(ntiles, per_sm * nsm);
     return launch_step(a, medium, limiter, kTile, kTile, 0, 0, grid, st) == cudaSuccess ? CLAW_OK : CLAW_ECUDA;
 }

@@ -208,17 +208,10 @@ template <int TX, int TY> struct Geo {
     static constexpr int QBYTES = 3 * QPL * 8;
     // shared-memory carve (in doubles), q buffers first (128-byte aligned)
     static constexpr int QSTRIDE = (3 * QPL + 15) / 16 * 16;
-    // rows a tile hands to the tile above it in a column walk (top rows of each array):
-    // x-edge strengths 2 rows, y-edge strengths 3, limited x-edges 2, limited y-edges 1, D 1
-    static constexpr int C_A = 0, C_B = 4 * XEW, C_S = C_B + 6 * YEW, C_SY = C_S + 4 * XLW,
-                         C_D = C_SY + 2 * YLW, NCARRY = C_D + DW;
     static constexpr int NWORK = 2 * XEW * XEH + 2 * YEW * YEH + 2 * XLW * XLH + 2 * YLW * YLH +
                                  DW * DH + EW * EH;
-    // q buffers, work arrays, 64 bytes of barriers, then (column walks only) the carried rows
-    static size_t smem_bytes(int nbuf, bool walk = false)
-    {
-        return (size_t)(nbuf * QSTRIDE + NWORK) * 8 + 64 + (walk ? (size_t)NCARRY * 8 : 0);
-    }
+    // q buffers, work arrays, 64 bytes of barriers
+    static size_t smem_bytes(int nbuf) { return (size_t)(nbuf * QSTRIDE + NWORK) * 8 + 64; }
 };
 
 // The tiles [*begin, *end) of CTA b of `grid` in a column walk: the contiguous range whose
@@ -399,24 +392,24 @@ __device__ __forceinline__ void pull_ghosts(const StepArgs& A, const PatchDev& P
 }
 
 // ------------------------------------------------------------------------- the kernel
-// MED: 0 uniform medium (rho0, K0), 1 cell-wise aux planes.
+// The cell-wise medium (aux planes; claw_step_uniform.cuh is the uniform medium's step).
 // STAGE: 0 cooperative loads, 1 tensor bulk copies (double buffered: the next tile streams in
 // during the whole of this one), 2 tensor bulk copies into one buffer (the next tile is requested
 // once this one's state has been read, in phase D) with registers capped for three CTAs per SM.
 // PULL: 1 same-level and boundary ghosts are taken from their source cells (a separate
 // instantiation: the mere presence of the pull code slowed the other kernels by up to 11 %);
 // 2 those and the ghosts interpolated from the coarser level, evaluated in the step.
-// REC (cell-wise medium): also write the step's intermediates to the tape A.tape (TapePlane);
+// REC: also write the step's intermediates to the tape A.tape (TapePlane);
 // each padded cell's entries come from the one tile that owns the cell (its interior, plus the
 // box's ghost frame next to it), so the tape is the same whatever the tiling.
+// The CTAs stride over the tiles by the grid (column walks are built for no cell-wise medium: its
+// ghost coefficients are the caller's and need not match the neighbour's interior).
 // Registers: the one-buffer staging is capped for three CTAs per SM; the 128-thread tiles for
 // five (the shared memory of five fits an SM), except those evaluating interpolated ghosts.
-template <int MED, int LIM, int TX, int TY, int NT, int STAGE, int PULL, bool REC = false>
+template <int LIM, int TX, int TY, int NT, int STAGE, int PULL, bool REC = false>
 __global__ void __launch_bounds__(NT, STAGE == 2 ? 3 : (NT == 128 && !REC ? 5 : 1))
     step_kernel(const StepArgs A)
 {
-    static_assert(!REC || MED == 1, "the tape records the cell-wise step");
-    // (REC kernels never walk: column walks are built for the uniform medium only)
     using G = Geo<TX, TY>;
     constexpr int NBUF = STAGE == 1 ? 2 : 1;
     constexpr int NPER = (TX * TY + NT - 1) / NT;
@@ -440,48 +433,22 @@ __global__ void __launch_bounds__(NT, STAGE == 2 ? 3 : (NT == 128 && !REC ? 5 : 
     double* Dx = Py + G::YLW * G::YLH;              // x-fluctuation pressure into each cell
     double* Ey = Dx + G::DW * G::DH;                // y-fluctuation pressure into each cell
     unsigned long long* bar = reinterpret_cast<unsigned long long*>(Ey + G::EW * G::EH);
-    // rows carried to the next tile of a column walk: allocated only for launches that walk
-    double* Cy = reinterpret_cast<double*>(bar) + 8;
     __shared__ unsigned long long s_tmax[2];   // per-tile speed max, double-buffered by tile parity
     __shared__ int s_flag;
-    __shared__ int s_range[2];                 // this CTA's tiles in a column walk
     __shared__ double s_k[16];                 // per-tile constants, written by thread 0
-    __shared__ double s_med[3];                // uniform medium Z0, c0, 1 / Z0, written by thread 0
 
     const int tid = threadIdx.x;
     if (tid == 0) {
         s_tmax[0] = s_tmax[1] = 0ull;
         s_flag = 0;
-        if (MED == 0) {   // square roots and a division: thread 0 alone (all threads cost ~0.9 FP64 per cell)
-            s_med[0] = sqrt(A.K0 * A.rho0);
-            s_med[1] = sqrt(A.K0 / A.rho0);
-            s_med[2] = 1.0 / s_med[0];
-        }
         if (STAGE) {
             mbar_init(&bar[0], 1);
             mbar_init(&bar[1], 1);
             fence_barrier_init();
         }
-        if (A.tcum) {
-            s_range[0] = walk_start(A.tcum, A.ntiles, blockIdx.x, nstep);
-            s_range[1] = walk_start(A.tcum, A.ntiles, blockIdx.x + 1, nstep);
-        } else {
-            s_range[0] = blockIdx.x;
-            s_range[1] = A.ntiles;
-        }
     }
     __syncthreads();
-    // Column walk (A.tcum set): the CTA takes a contiguous range of tiles, and a tile flagged
-    // TILE_CARRY that follows its lower neighbour in the same range takes the rows the two share
-    // (edges of the rows between them) from that neighbour instead of recomputing them: the
-    // neighbour is the tile directly below in the same box or (uniform medium) in the same-level
-    // box below, whose shared rows hold the same values.  Otherwise the CTA strides over all
-    // tiles by the grid.
-    // Only the uniform medium walks (the host builds column walks for no other kind), so the
-    // cell-wise kernels carry none of this code.
-    const int t_begin = s_range[0], t_end = s_range[1];
-    const int t_step = A.tcum ? 1 : nstep;
-    const bool walk = MED == 0 && A.tcum != nullptr;
+    const int t_end = A.ntiles, t_step = nstep;
 
     const CUtensorMap* tmaps = reinterpret_cast<const CUtensorMap*>(A.tmaps);
     int my_flag = 0;
@@ -493,29 +460,18 @@ __global__ void __launch_bounds__(NT, STAGE == 2 ? 3 : (NT == 128 && !REC ? 5 : 
         if (cur_run >= 0 && cur_max)
             atomicMax(reinterpret_cast<unsigned long long*>(A.smax) + cur_run, cur_max);
     };
-    // uniform medium constants (once per CTA)
-    double Z0 = 0, c0 = 0, iZ = 0;
-    if (MED == 0) {
-        Z0 = s_med[0];
-        c0 = s_med[1];
-        iZ = s_med[2];
-    }
 
     auto issue = [&](int t, int b) {
         const TileDev T = A.tiles[t];
         mbar_expect_tx(&bar[b], (unsigned)G::QBYTES);
         tma_load_3d(qbuf + b * G::QSTRIDE, &tmaps[T.patch], T.x0, T.y0, 0, &bar[b]);
     };
-    if (STAGE && tid == 0 && t_begin < t_end) issue(t_begin, 0);
+    if (STAGE && tid == 0 && (int)blockIdx.x < t_end) issue(blockIdx.x, 0);
 
     int it = 0;
-    for (int t = t_begin; t < t_end; t += t_step, ++it) {
+    for (int t = blockIdx.x; t < t_end; t += t_step, ++it) {
         const int b = STAGE == 1 ? (it & 1) : 0;
         const TileDev T = A.tiles[t];
-        // carry: this tile's lowest rows come from the previous tile; hand: the next one takes
-        // this tile's top rows
-        const bool carry = walk && t > t_begin && (T.flags & TILE_CARRY);
-        const bool hand = walk && t + 1 < t_end && (A.tiles[t + 1].flags & TILE_CARRY);
         const PatchDev P = A.patches[T.patch];
         const int tx = T.tx, ty = T.ty, x0 = T.x0, y0 = T.y0;
         const int W = P.nx + 4;
@@ -574,28 +530,9 @@ __global__ void __launch_bounds__(NT, STAGE == 2 ? 3 : (NT == 128 && !REC ? 5 : 
             s_k[13] = ly;
             s_k[14] = -0.5 * lx;
             s_k[15] = -0.5 * ly;
-            if (MED == 0) {
-                // the centre part 2 kT (D + E) of the transverse pressure update folds into the
-                // normal-update coefficients (D = ap + kDx bp, E likewise); phase D adds the rest
-                const double kapx = c0 * (1.0 - lx * c0), kapy = c0 * (1.0 - ly * c0);
-                const double kDx = cw ? 1.0 - lx * c0 : 0.0, kDy = cw ? 1.0 - ly * c0 : 0.0;
-                const double kT = trans ? 0.125 * lx * ly * c0 * A.K0 : 0.0;
-                s_k[0] = fma(-0.5 * lx, A.K0, 2.0 * kT);              // cpa
-                s_k[1] = fma(-0.25 * lx * kapx, Z0, 2.0 * kT * kDx);  // cpb
-                s_k[2] = -0.5 * lx * c0;                              // cua
-                s_k[3] = -0.25 * lx * kapx;                           // cub
-                s_k[4] = fma(-0.5 * ly, A.K0, 2.0 * kT);              // cpay
-                s_k[5] = fma(-0.25 * ly * kapy, Z0, 2.0 * kT * kDy);  // cpby
-                s_k[6] = -0.5 * ly * c0;                              // cva
-                s_k[7] = -0.25 * ly * kapy;                           // cvb
-                s_k[8] = kDx;
-                s_k[9] = kDy;
-                s_k[10] = -kT;
-                s_k[11] = trans ? 0.125 * lx * ly * c0 * c0 : 0.0;   // kU
-            }
         }
-        // medium access (MED == 1): aux plane k of the cell at tile-local (i, j)
-        const double* aux = MED ? A.aux + P.aoff : nullptr;
+        // medium access: aux plane k of the cell at tile-local (i, j)
+        const double* aux = A.aux + P.aoff;
         auto AX = [&](int k, int i, int j) -> double {
             return __ldg(aux + k * WH + (long long)(y0 + j + 2) * W + (x0 + i + 2));
         };
@@ -609,74 +546,45 @@ __global__ void __launch_bounds__(NT, STAGE == 2 ? 3 : (NT == 128 && !REC ? 5 : 
         };
 
         // ---------------------------------------------------------------- phase A: normal Riemann
-        // carried rows land in the lowest rows of the arrays, which this phase does not write
-        // (the previous tile's last reads of them were behind its end-of-tile barrier)
-        if (carry) {
-            for (int k = tid; k < G::NCARRY; k += NT) {
-                double* dst;
-                if (k < G::C_B) dst = k < 2 * G::XEW ? A1x + k : A2x + (k - 2 * G::XEW);
-                else if (k < G::C_S) dst = k < G::C_B + 3 * G::YEW ? B1y + (k - G::C_B) : B2y + (k - G::C_B - 3 * G::YEW);
-                else if (k < G::C_SY) dst = k < G::C_S + 2 * G::XLW ? Sx + (k - G::C_S) : Px + (k - G::C_S - 2 * G::XLW);
-                else if (k < G::C_D) dst = k < G::C_SY + G::YLW ? Sy + (k - G::C_SY) : Py + (k - G::C_SY - G::YLW);
-                else dst = Dx + (k - G::C_D);
-                *dst = Cy[k];
-            }
-        }
-        // first rows computed here: with a carry, the rows below come from the previous tile
-        const int rx0 = carry ? 1 : -1;   // x-edges and limited x-edges: rows [rx0, ty]
-        const int by0 = carry ? 2 : -1;   // y-edges: b in [by0, ty + 1]
-        const int ly0 = carry ? 1 : 0;    // limited y-edges: b in [ly0, ty]
         // x-edge a (between cells a-1 and a) on rows r in [-1, ty]
         {
-            const int w = tx + 3, n = (ty + 1 - rx0) * w;
+            const int w = tx + 3, n = (ty + 2) * w;
             for (int k = tid; k < n; k += NT) {
-                const int r = k / w + rx0, a = k - (r - rx0) * w - 1;
+                const int r = k / w - 1, a = k - (r + 1) * w - 1;
                 const int iR = (a + 2) + (r + 2) * G::SW;
                 const double dp = sp[iR] - sp[iR - 1];
                 const double du = su[iR] - su[iR - 1];
                 double a1, a2;
-                if (MED == 0) {   // 2 alpha: du -/+ dp / Z
-                    a1 = fma(-dp, iZ, du);
-                    a2 = fma(dp, iZ, du);
-                } else {
-                    const double zr = AX(AUX_Z, a, r), zl = AX(AUX_Z, a - 1, r), is = AX(AUX_IXS, a, r);
-                    a1 = fma(zr, du, -dp) * is;
-                    a2 = fma(zl, du, dp) * is;
-                    rec(TAPE_A1, a, r, a1);
-                    rec(TAPE_A2, a, r, a2);
-                }
+                const double zr = AX(AUX_Z, a, r), zl = AX(AUX_Z, a - 1, r), is = AX(AUX_IXS, a, r);
+                a1 = fma(zr, du, -dp) * is;
+                a2 = fma(zl, du, dp) * is;
+                rec(TAPE_A1, a, r, a1);
+                rec(TAPE_A2, a, r, a2);
                 A1x[(r + 1) * G::XEW + (a + 1)] = a1;
                 A2x[(r + 1) * G::XEW + (a + 1)] = a2;
             }
         }
         // y-edge b (between rows b-1 and b) on columns c in [-1, tx]
         {
-            const int w = tx + 2, n = (ty + 2 - by0) * w;
+            const int w = tx + 2, n = (ty + 3) * w;
             for (int k = tid; k < n; k += NT) {
-                const int bb = k / w + by0, c = k - (bb - by0) * w - 1;
+                const int bb = k / w - 1, c = k - (bb + 1) * w - 1;
                 const int iR = (c + 2) + (bb + 2) * G::SW;
                 const double dp = sp[iR] - sp[iR - G::SW];
                 const double dv = sv[iR] - sv[iR - G::SW];
                 double b1, b2;
-                if (MED == 0) {
-                    b1 = fma(-dp, iZ, dv);
-                    b2 = fma(dp, iZ, dv);
-                } else {
-                    const double zr = AX(AUX_Z, c, bb), zl = AX(AUX_Z, c, bb - 1), is = AX(AUX_IYS, c, bb);
-                    b1 = fma(zr, dv, -dp) * is;
-                    b2 = fma(zl, dv, dp) * is;
-                    rec(TAPE_B1, c, bb, b1);
-                    rec(TAPE_B2, c, bb, b2);
-                }
+                const double zr = AX(AUX_Z, c, bb), zl = AX(AUX_Z, c, bb - 1), is = AX(AUX_IYS, c, bb);
+                b1 = fma(zr, dv, -dp) * is;
+                b2 = fma(zl, dv, dp) * is;
+                rec(TAPE_B1, c, bb, b1);
+                rec(TAPE_B2, c, bb, b2);
                 B1y[(bb + 1) * G::YEW + (c + 1)] = b1;
                 B2y[(bb + 1) * G::YEW + (c + 1)] = b2;
             }
         }
         // wave speeds seen by this tile (ring [-1,tx] x [-1,ty]): integer max of bit patterns,
         // warp shuffle, shared atomic
-        if (MED == 0) {
-            if (tid == 0) s_tmax[it & 1] = (unsigned long long)__double_as_longlong(c0);
-        } else {
+        {
             unsigned long long m = 0ull;
             const int w = tx + 2, n = (ty + 2) * w;
             for (int k = tid; k < n; k += NT) {
@@ -693,90 +601,58 @@ __global__ void __launch_bounds__(NT, STAGE == 2 ? 3 : (NT == 128 && !REC ? 5 : 
         const double lx = s_k[12], ly = s_k[13];
         if (second) {
             {
-                const int w = tx + 1, n = (ty + 1 - rx0) * w;
+                const int w = tx + 1, n = (ty + 2) * w;
                 for (int k = tid; k < n; k += NT) {
-                    const int r = k / w + rx0, a = k - (r - rx0) * w;
+                    const int r = k / w - 1, a = k - (r + 1) * w;
                     const int e = (r + 1) * G::XEW + (a + 1);
                     const double a1 = A1x[e], a2 = A2x[e];
                     double m1, m2;
-                    if (MED == 0) {
-                        m1 = Lim<LIM>::f(a1, A1x[e + 1]);   // left-going: upwind edge a+1
-                        m2 = Lim<LIM>::f(a2, A2x[e - 1]);   // right-going: upwind edge a-1
-                        Sx[(r + 1) * G::XLW + a] = m2 - m1;
-                        Px[(r + 1) * G::XLW + a] = m1 + m2;
+                    if (REC) {
+                        int c1, c2;
+                        m1 = Lim<LIM>::template fc<true>(a1, A1x[e + 1] * AX(AUX_FX1, a, r), c1);
+                        m2 = Lim<LIM>::template fc<true>(a2, A2x[e - 1] * AX(AUX_FX2, a, r), c2);
+                        rec(TAPE_M1, a, r, tag_code(m1, c1));
+                        rec(TAPE_M2, a, r, tag_code(m2, c2));
                     } else {
-                        if (REC) {
-                            int c1, c2;
-                            m1 = Lim<LIM>::template fc<true>(a1, A1x[e + 1] * AX(AUX_FX1, a, r), c1);
-                            m2 = Lim<LIM>::template fc<true>(a2, A2x[e - 1] * AX(AUX_FX2, a, r), c2);
-                            rec(TAPE_M1, a, r, tag_code(m1, c1));
-                            rec(TAPE_M2, a, r, tag_code(m2, c2));
-                        } else {
-                            m1 = Lim<LIM>::template f<true>(a1, A1x[e + 1] * AX(AUX_FX1, a, r));
-                            m2 = Lim<LIM>::template f<true>(a2, A2x[e - 1] * AX(AUX_FX2, a, r));
-                        }
-                        const double kl = fma(-lx, AX(AUX_C2, a - 1, r), AX(AUX_C, a - 1, r));
-                        const double kr = fma(-lx, AX(AUX_C2, a, r), AX(AUX_C, a, r));
-                        const double e1 = kl * m1, e2 = kr * m2;
-                        Sx[(r + 1) * G::XLW + a] = fma(AX(AUX_Z, a, r), e2, -(AX(AUX_Z, a - 1, r) * e1));
-                        Px[(r + 1) * G::XLW + a] = e1 + e2;
+                        m1 = Lim<LIM>::template f<true>(a1, A1x[e + 1] * AX(AUX_FX1, a, r));
+                        m2 = Lim<LIM>::template f<true>(a2, A2x[e - 1] * AX(AUX_FX2, a, r));
                     }
+                    const double kl = fma(-lx, AX(AUX_C2, a - 1, r), AX(AUX_C, a - 1, r));
+                    const double kr = fma(-lx, AX(AUX_C2, a, r), AX(AUX_C, a, r));
+                    const double e1 = kl * m1, e2 = kr * m2;
+                    Sx[(r + 1) * G::XLW + a] = fma(AX(AUX_Z, a, r), e2, -(AX(AUX_Z, a - 1, r) * e1));
+                    Px[(r + 1) * G::XLW + a] = e1 + e2;
                 }
             }
             {
-                const int w = tx + 2, n = (ty + 1 - ly0) * w;
+                const int w = tx + 2, n = (ty + 1) * w;
                 for (int k = tid; k < n; k += NT) {
-                    const int bb = k / w + ly0, c = k - (bb - ly0) * w - 1;
+                    const int bb = k / w, c = k - bb * w - 1;
                     const int e = (bb + 1) * G::YEW + (c + 1);
                     const double b1 = B1y[e], b2 = B2y[e];
                     double m1, m2;
-                    if (MED == 0) {
-                        m1 = Lim<LIM>::f(b1, B1y[e + G::YEW]);
-                        m2 = Lim<LIM>::f(b2, B2y[e - G::YEW]);
-                        Sy[bb * G::YLW + (c + 1)] = m2 - m1;
-                        Py[bb * G::YLW + (c + 1)] = m1 + m2;
+                    if (REC) {
+                        int c1, c2;
+                        m1 = Lim<LIM>::template fc<true>(b1, B1y[e + G::YEW] * AX(AUX_FY1, c, bb), c1);
+                        m2 = Lim<LIM>::template fc<true>(b2, B2y[e - G::YEW] * AX(AUX_FY2, c, bb), c2);
+                        rec(TAPE_N1, c, bb, tag_code(m1, c1));
+                        rec(TAPE_N2, c, bb, tag_code(m2, c2));
                     } else {
-                        if (REC) {
-                            int c1, c2;
-                            m1 = Lim<LIM>::template fc<true>(b1, B1y[e + G::YEW] * AX(AUX_FY1, c, bb), c1);
-                            m2 = Lim<LIM>::template fc<true>(b2, B2y[e - G::YEW] * AX(AUX_FY2, c, bb), c2);
-                            rec(TAPE_N1, c, bb, tag_code(m1, c1));
-                            rec(TAPE_N2, c, bb, tag_code(m2, c2));
-                        } else {
-                            m1 = Lim<LIM>::template f<true>(b1, B1y[e + G::YEW] * AX(AUX_FY1, c, bb));
-                            m2 = Lim<LIM>::template f<true>(b2, B2y[e - G::YEW] * AX(AUX_FY2, c, bb));
-                        }
-                        const double kl = fma(-ly, AX(AUX_C2, c, bb - 1), AX(AUX_C, c, bb - 1));
-                        const double kr = fma(-ly, AX(AUX_C2, c, bb), AX(AUX_C, c, bb));
-                        const double e1 = kl * m1, e2 = kr * m2;
-                        Sy[bb * G::YLW + (c + 1)] = fma(AX(AUX_Z, c, bb), e2, -(AX(AUX_Z, c, bb - 1) * e1));
-                        Py[bb * G::YLW + (c + 1)] = e1 + e2;
+                        m1 = Lim<LIM>::template f<true>(b1, B1y[e + G::YEW] * AX(AUX_FY1, c, bb));
+                        m2 = Lim<LIM>::template f<true>(b2, B2y[e - G::YEW] * AX(AUX_FY2, c, bb));
                     }
+                    const double kl = fma(-ly, AX(AUX_C2, c, bb - 1), AX(AUX_C, c, bb - 1));
+                    const double kr = fma(-ly, AX(AUX_C2, c, bb), AX(AUX_C, c, bb));
+                    const double e1 = kl * m1, e2 = kr * m2;
+                    Sy[bb * G::YLW + (c + 1)] = fma(AX(AUX_Z, c, bb), e2, -(AX(AUX_Z, c, bb - 1) * e1));
+                    Py[bb * G::YLW + (c + 1)] = e1 + e2;
                 }
             }
             __syncthreads();
         }
 
         // ---------------------------------------------------------------- phase C: per-cell terms
-        // uniform medium, with a = 2 alpha and M = phi(theta) a:
-        //   x-normal update  dp = -(lx K/2) ap - (lx kap Z/4) bp,  du = -(lx c/2) au - (lx kap/4) bu
-        //   (dp also carries the centre term 2 kT D of the transverse update)
-        //   ap = A2_w + A1_e, au = A2_w - A1_e, bp = S_e - S_w, bu = P_e - P_w,  kap = c (1 - lx c)
-        //   x-fluctuation pressure into the cell D = (K/2) (ap + (1 - lx c) bp)
         // cell-wise medium: D = K ap + bp,  x-normal (K ap + bp/2, c au + bu/2)
-        double cpa = 0, cpb = 0, cua = 0, cub = 0, cpay = 0, cpby = 0, cva = 0, cvb = 0, kDx = 0, kDy = 0;
-        if (MED == 0) {
-            cpa = s_k[0];
-            cpb = s_k[1];
-            cua = s_k[2];
-            cub = s_k[3];
-            cpay = s_k[4];
-            cpby = s_k[5];
-            cva = s_k[6];
-            cvb = s_k[7];
-            kDx = s_k[8];
-            kDy = s_k[9];
-        }
         // dP, dU, dV: Q plus the normal updates (the transverse terms are added in phase D)
         double dP[NPER], dU[NPER], dV[NPER];
 #pragma unroll
@@ -797,47 +673,34 @@ __global__ void __launch_bounds__(NT, STAGE == 2 ? 3 : (NT == 128 && !REC ? 5 : 
                 bpy = Sy[(r + 1) * G::YLW + c + 1] - Sy[r * G::YLW + c + 1];
                 bvy = Py[(r + 1) * G::YLW + c + 1] - Py[r * G::YLW + c + 1];
             }
-            if (MED == 0) {
-                if (trans) {
-                    Dx[(r + 1) * G::DW + c] = fma(kDx, bpx, apx);
-                    Ey[r * G::EW + c + 1] = fma(kDy, bpy, apy);
-                }
-                dP[n] = fma(cpa, apx, fma(cpb, bpx, fma(cpay, apy, fma(cpby, bpy, sp[iq]))));
-                dU[n] = fma(cua, aux_, fma(cub, bux, su[iq]));
-                dV[n] = fma(cva, avy, fma(cvb, bvy, sv[iq]));
-            } else {
-                const double Kc = AX(AUX_K, c, r), cc = AX(AUX_C, c, r);
-                if (trans) {
-                    const double dd = cw ? fma(Kc, apx, bpx) : Kc * apx;
-                    const double ee = cw ? fma(Kc, apy, bpy) : Kc * apy;
-                    Dx[(r + 1) * G::DW + c] = dd;
-                    Ey[r * G::EW + c + 1] = ee;
-                    rec(TAPE_D, c, r, dd);
-                    rec(TAPE_E, c, r, ee);
-                }
-                const double tpx = fma(0.5, bpx, Kc * apx), tux = fma(0.5, bux, cc * aux_);
-                const double tpy = fma(0.5, bpy, Kc * apy), tvy = fma(0.5, bvy, cc * avy);
-                dP[n] = fma(-lx, tpx, fma(-ly, tpy, sp[iq]));
-                dU[n] = fma(-lx, tux, su[iq]);
-                dV[n] = fma(-ly, tvy, sv[iq]);
+            const double Kc = AX(AUX_K, c, r), cc = AX(AUX_C, c, r);
+            if (trans) {
+                const double dd = cw ? fma(Kc, apx, bpx) : Kc * apx;
+                const double ee = cw ? fma(Kc, apy, bpy) : Kc * apy;
+                Dx[(r + 1) * G::DW + c] = dd;
+                Ey[r * G::EW + c + 1] = ee;
+                rec(TAPE_D, c, r, dd);
+                rec(TAPE_E, c, r, ee);
             }
+            const double tpx = fma(0.5, bpx, Kc * apx), tux = fma(0.5, bux, cc * aux_);
+            const double tpy = fma(0.5, bpy, Kc * apy), tvy = fma(0.5, bvy, cc * avy);
+            dP[n] = fma(-lx, tpx, fma(-ly, tpy, sp[iq]));
+            dU[n] = fma(-lx, tux, su[iq]);
+            dV[n] = fma(-ly, tvy, sv[iq]);
         }
         // D on the ghost rows -1, ty and E on the ghost columns -1, tx (transverse only)
         if (trans) {
             const int n = 2 * (tx + ty);
-            for (int k = tid + (carry ? tx : 0); k < n; k += NT) {   // row -1 is carried
+            for (int k = tid; k < n; k += NT) {
                 if (k < 2 * tx) {
                     const int c = k % tx, r = (k < tx) ? -1 : ty;
                     const int ex = (r + 1) * G::XEW + (c + 1);
                     const double apx = A2x[ex] + A1x[ex + 1];
                     const double bpx = second ? Sx[(r + 1) * G::XLW + c + 1] - Sx[(r + 1) * G::XLW + c] : 0.0;
                     double d;
-                    if (MED == 0) d = fma(kDx, bpx, apx);
-                    else {
-                        const double Kc = AX(AUX_K, c, r);
-                        d = cw ? fma(Kc, apx, bpx) : Kc * apx;
-                        rec(TAPE_D, c, r, d);
-                    }
+                    const double Kc = AX(AUX_K, c, r);
+                    d = cw ? fma(Kc, apx, bpx) : Kc * apx;
+                    rec(TAPE_D, c, r, d);
                     Dx[(r + 1) * G::DW + c] = d;
                 } else {
                     const int kk = k - 2 * tx;
@@ -846,30 +709,11 @@ __global__ void __launch_bounds__(NT, STAGE == 2 ? 3 : (NT == 128 && !REC ? 5 : 
                     const double apy = B2y[ey] + B1y[ey + G::YEW];
                     const double bpy = second ? Sy[(r + 1) * G::YLW + c + 1] - Sy[r * G::YLW + c + 1] : 0.0;
                     double e;
-                    if (MED == 0) e = fma(kDy, bpy, apy);
-                    else {
-                        const double Kc = AX(AUX_K, c, r);
-                        e = cw ? fma(Kc, apy, bpy) : Kc * apy;
-                        rec(TAPE_E, c, r, e);
-                    }
+                    const double Kc = AX(AUX_K, c, r);
+                    e = cw ? fma(Kc, apy, bpy) : Kc * apy;
+                    rec(TAPE_E, c, r, e);
                     Ey[r * G::EW + c + 1] = e;
                 }
-            }
-        }
-        // hand the top rows of the edge arrays to the next tile (none of them is written from
-        // here to the end of the tile, but phase C2 reuses the strength arrays)
-        if (hand) {
-            for (int k = tid; k < G::C_D; k += NT) {
-                const double* src;
-                if (k < G::C_B) src = k < 2 * G::XEW ? A1x + ty * G::XEW + k : A2x + ty * G::XEW + (k - 2 * G::XEW);
-                else if (k < G::C_S)
-                    src = k < G::C_B + 3 * G::YEW ? B1y + ty * G::YEW + (k - G::C_B)
-                                                  : B2y + ty * G::YEW + (k - G::C_B - 3 * G::YEW);
-                else if (k < G::C_SY)
-                    src = k < G::C_S + 2 * G::XLW ? Sx + ty * G::XLW + (k - G::C_S)
-                                                  : Px + ty * G::XLW + (k - G::C_S - 2 * G::XLW);
-                else src = k < G::C_SY + G::YLW ? Sy + ty * G::YLW + (k - G::C_SY) : Py + ty * G::YLW + (k - G::C_SY - G::YLW);
-                Cy[k] = *src;
             }
         }
         __syncthreads();
@@ -881,7 +725,7 @@ __global__ void __launch_bounds__(NT, STAGE == 2 ? 3 : (NT == 128 && !REC ? 5 : 
         double* Gv = B2y;
         double* Fp = A1x;
         double* Fu = A2x;
-        if (MED == 1 && trans) {
+        if (trans) {
             {   // y-edge jj in [0, ty] of column c in [0, tx): lo = (c, jj-1), hi = (c, jj)
                 const int n = (ty + 1) * tx;
                 for (int k = tid; k < n; k += NT) {
@@ -913,14 +757,6 @@ __global__ void __launch_bounds__(NT, STAGE == 2 ? 3 : (NT == 128 && !REC ? 5 : 
         // one staging buffer: the tile's state was last read in phase C (behind the barrier
         // above), so the next tile's copy can land while this one finishes
         if (STAGE == 2 && tid == 0 && t + t_step < t_end) issue(t + t_step, 0);
-        double kT = 0, kU = 0;
-        if (MED == 0 && trans) {
-            kT = s_k[10];
-            kU = s_k[11];
-        }
-        // D of row ty - 1 becomes the next tile's row -1 (final since the barrier ending phase C)
-        if (hand)
-            for (int k = tid; k < G::DW; k += NT) Cy[G::C_D + k] = Dx[ty * G::DW + k];
         double* dst = A.qnew + P.qoff;
 #pragma unroll
         for (int n = 0; n < NPER; ++n) {
@@ -929,19 +765,11 @@ __global__ void __launch_bounds__(NT, STAGE == 2 ? 3 : (NT == 128 && !REC ? 5 : 
             if (ci >= TX * TY || c >= tx || r >= ty) continue;
             double p = dP[n], u = dU[n], v = dV[n];
             if (trans) {
-                if (MED == 0) {
-                    const double dn = Dx[(r + 2) * G::DW + c], ds = Dx[r * G::DW + c];
-                    const double ee = Ey[r * G::EW + c + 2], ew = Ey[r * G::EW + c];
-                    p = fma(kT, (dn + ds) + (ee + ew), p);   // kT holds -kT; 2 kT (dc + ec) is in p
-                    u = fma(kU, ee - ew, u);
-                    v = fma(kU, dn - ds, v);
-                } else {
-                    const double fpe = Fp[r * (TX + 1) + c + 1], fpw = Fp[r * (TX + 1) + c];
-                    const double gpn = Gp[(r + 1) * TX + c], gps = Gp[r * TX + c];
-                    p = fma(-lx, fpe - fpw, fma(-ly, gpn - gps, p));
-                    u = fma(-lx, Fu[r * (TX + 1) + c + 1] - Fu[r * (TX + 1) + c], u);
-                    v = fma(-ly, Gv[(r + 1) * TX + c] - Gv[r * TX + c], v);
-                }
+                const double fpe = Fp[r * (TX + 1) + c + 1], fpw = Fp[r * (TX + 1) + c];
+                const double gpn = Gp[(r + 1) * TX + c], gps = Gp[r * TX + c];
+                p = fma(-lx, fpe - fpw, fma(-ly, gpn - gps, p));
+                u = fma(-lx, Fu[r * (TX + 1) + c + 1] - Fu[r * (TX + 1) + c], u);
+                v = fma(-ly, Gv[(r + 1) * TX + c] - Gv[r * TX + c], v);
             }
             if (not_finite(p) | not_finite(u) | not_finite(v)) my_flag |= ERR_NAN;
             const long long o = (long long)(y0 + r + 2) * W + (x0 + c + 2);
@@ -978,53 +806,51 @@ namespace claw {
 // kernel pointer and dynamic shared memory of one configuration
 struct StepKernel {
     void (*fn)(const StepArgs);
-    size_t smem;        // dynamic shared memory of a launch that strides over the tiles
+    size_t smem;        // dynamic shared memory of a launch
     int nt;
-    size_t smem_walk;   // ... of a launch that walks tile columns (the carried rows added)
+    size_t smem_walk;   // ... of a launch that walks tile columns (shallow water: carried rows added)
 };
 
-template <int MED, int LIM, int TX, int TY, int NT, int STAGE, int PULL, bool REC = false>
+template <int LIM, int TX, int TY, int NT, int STAGE, int PULL, bool REC = false>
 StepKernel step_kernel_entry()
 {
     StepKernel k;
-    k.fn = step_kernel<MED, LIM, TX, TY, NT, STAGE, PULL, REC>;
-    k.smem = Geo<TX, TY>::smem_bytes(STAGE == 1 ? 2 : 1);
+    k.fn = step_kernel<LIM, TX, TY, NT, STAGE, PULL, REC>;
+    k.smem = k.smem_walk = Geo<TX, TY>::smem_bytes(STAGE == 1 ? 2 : 1);
     k.nt = NT;
-    k.smem_walk = MED == 1 ? k.smem : Geo<TX, TY>::smem_bytes(STAGE == 1 ? 2 : 1, true);
     return k;
 }
 
-// all tile shapes and stagings of one medium and limiter
-// tile shapes x thread counts x stagings of one medium and limiter (nt = 0: the default)
-template <int MED, int LIM, int PULL, bool REC = false>
+// tile shapes x thread counts x stagings of one limiter, cell-wise medium (nt = 0: the default)
+template <int LIM, int PULL, bool REC = false>
 StepKernel step_kernel_select(int tx, int ty, int nt, int staging)
 {
     if (tx == 32 && ty == 32 && (nt == 0 || nt == 256))
-        return staging ? step_kernel_entry<MED, LIM, 32, 32, 256, 1, PULL, REC>()
-                       : step_kernel_entry<MED, LIM, 32, 32, 256, 0, PULL, REC>();
+        return staging ? step_kernel_entry<LIM, 32, 32, 256, 1, PULL, REC>()
+                       : step_kernel_entry<LIM, 32, 32, 256, 0, PULL, REC>();
     if (tx == 32 && ty == 32 && nt == 512)
-        return staging ? step_kernel_entry<MED, LIM, 32, 32, 512, 1, PULL, REC>()
-                       : step_kernel_entry<MED, LIM, 32, 32, 512, 0, PULL, REC>();
+        return staging ? step_kernel_entry<LIM, 32, 32, 512, 1, PULL, REC>()
+                       : step_kernel_entry<LIM, 32, 32, 512, 0, PULL, REC>();
     if (tx == 32 && ty == 16 && (nt == 0 || nt == 256)) {
-        if (staging == 2) return step_kernel_entry<MED, LIM, 32, 16, 256, 2, PULL, REC>();
-        return staging ? step_kernel_entry<MED, LIM, 32, 16, 256, 1, PULL, REC>()
-                       : step_kernel_entry<MED, LIM, 32, 16, 256, 0, PULL, REC>();
+        if (staging == 2) return step_kernel_entry<LIM, 32, 16, 256, 2, PULL, REC>();
+        return staging ? step_kernel_entry<LIM, 32, 16, 256, 1, PULL, REC>()
+                       : step_kernel_entry<LIM, 32, 16, 256, 0, PULL, REC>();
     }
     if (tx == 16 && ty == 16 && (nt == 0 || nt == 128))
-        return staging ? step_kernel_entry<MED, LIM, 16, 16, 128, 1, PULL, REC>()
-                       : step_kernel_entry<MED, LIM, 16, 16, 128, 0, PULL, REC>();
+        return staging ? step_kernel_entry<LIM, 16, 16, 128, 1, PULL, REC>()
+                       : step_kernel_entry<LIM, 16, 16, 128, 0, PULL, REC>();
     return StepKernel{nullptr, 0, 0, 0};
 }
 
-template <int MED, int PULL, bool REC = false>
+template <int PULL, bool REC = false>
 StepKernel step_kernel_for(int lim, int tx, int ty, int nt, int staging)
 {
     switch (lim) {
-    case CLAW_LIM_NONE: return step_kernel_select<MED, CLAW_LIM_NONE, PULL, REC>(tx, ty, nt, staging);
-    case CLAW_LIM_MINMOD: return step_kernel_select<MED, CLAW_LIM_MINMOD, PULL, REC>(tx, ty, nt, staging);
-    case CLAW_LIM_SUPERBEE: return step_kernel_select<MED, CLAW_LIM_SUPERBEE, PULL, REC>(tx, ty, nt, staging);
-    case CLAW_LIM_VANLEER: return step_kernel_select<MED, CLAW_LIM_VANLEER, PULL, REC>(tx, ty, nt, staging);
-    case CLAW_LIM_MC: return step_kernel_select<MED, CLAW_LIM_MC, PULL, REC>(tx, ty, nt, staging);
+    case CLAW_LIM_NONE: return step_kernel_select<CLAW_LIM_NONE, PULL, REC>(tx, ty, nt, staging);
+    case CLAW_LIM_MINMOD: return step_kernel_select<CLAW_LIM_MINMOD, PULL, REC>(tx, ty, nt, staging);
+    case CLAW_LIM_SUPERBEE: return step_kernel_select<CLAW_LIM_SUPERBEE, PULL, REC>(tx, ty, nt, staging);
+    case CLAW_LIM_VANLEER: return step_kernel_select<CLAW_LIM_VANLEER, PULL, REC>(tx, ty, nt, staging);
+    case CLAW_LIM_MC: return step_kernel_select<CLAW_LIM_MC, PULL, REC>(tx, ty, nt, staging);
     }
     return StepKernel{nullptr, 0, 0, 0};
 }

@@ -5,6 +5,6 @@
 namespace claw {
 StepKernel step_kernel_cellwise_interp(int lim, int tx, int ty, int nt, int staging)
 {
-    return step_kernel_for<1, 2>(lim, tx, ty, nt, staging);
+    return step_kernel_for<2>(lim, tx, ty, nt, staging);
 }
 }  // namespace claw

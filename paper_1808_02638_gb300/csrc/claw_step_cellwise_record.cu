@@ -5,6 +5,6 @@
 namespace claw {
 StepKernel step_kernel_cellwise_record(int lim, int tx, int ty, int nt, int staging)
 {
-    return step_kernel_for<1, 1, true>(lim, tx, ty, nt, staging);
+    return step_kernel_for<1, true>(lim, tx, ty, nt, staging);
 }
 }  // namespace claw

@@ -1,10 +1,10 @@
 // Instantiations of the fused level-step (uniform medium) that pull the same-level and boundary ghosts
 // and evaluate the ghosts interpolated from the coarser level inside the step.
-#include "claw_step.cuh"
+#include "claw_step_uniform.cuh"
 
 namespace claw {
 StepKernel step_kernel_uniform_interp(int lim, int tx, int ty, int nt, int staging)
 {
-    return step_kernel_for<0, 2>(lim, tx, ty, nt, staging);
+    return uniform_kernel_for<2>(lim, tx, ty, nt, staging);
 }
 }  // namespace claw

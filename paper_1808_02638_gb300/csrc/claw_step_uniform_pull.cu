@@ -1,9 +1,9 @@
 // Instantiations of the fused level-step for a uniform medium that take pulled ghosts.
-#include "claw_step.cuh"
+#include "claw_step_uniform.cuh"
 
 namespace claw {
 StepKernel step_kernel_uniform_pull(int lim, int tx, int ty, int nt, int staging)
 {
-    return step_kernel_for<0, 1>(lim, tx, ty, nt, staging);
+    return uniform_kernel_for<1>(lim, tx, ty, nt, staging);
 }
 }  // namespace claw

@@ -128,11 +128,7 @@ static void column_walks(const LevelDev& d, int piece, std::vector<TileDev>& out
 }
 
 // tiles of a level for its tiling: sorted by area (largest first) for the persistent CTAs, or
-// as column walks (d.walk; automatic: acoustics levels with at least kWalkTilesPerSM tiles per
-// SM, where each CTA has several tiles to walk; with about one tile per CTA the area-sorted
-// stride balances better), and grouped by box for the per-box launches
-constexpr int kWalkTilesPerSM = 8;
-
+// as column walks (d.walk), and grouped by box for the per-box launches
 int build_tiles(claw_ctx* ctx, int L)
 {
     LevelDev& d = ctx->lev[L];
@@ -159,11 +155,10 @@ int build_tiles(claw_ctx* ctx, int L)
     pack.add(&ctx->ptiles[L], t);
     ctx->ptile_start[L] = start;
     d.htcum.clear();
-    // automatic: uniform-medium acoustics only (the shallow-water step issues 6 % fewer FP64
-    // instructions with walks but ran 1.5 % slower on the 2048^2 workload, with two CTAs per SM)
-    d.walking = ctx->kind() != KIND_CELLWISE &&
-                (d.walk > 0 || (d.walk < 0 && ctx->kind() == KIND_UNIFORM &&
-                                (long long)t.size() >= (long long)kWalkTilesPerSM * std::max(ctx->nsm, 1)));
+    // on request only: the uniform-medium step carries nothing from tile to tile, and walking (the
+    // same tiles in another order) took 262 against 244 us a step of 2048^2; the shallow-water step
+    // issues 6 % fewer FP64 instructions with walks but ran 1.5 % slower there
+    d.walking = ctx->kind() != KIND_CELLWISE && d.walk > 0;
     if (d.walking) {
         // pieces of about the tiles one CTA takes (three CTAs per SM, a guess: the launch picks
         // its grid later), at least 4 and at most 64

@@ -18,12 +18,18 @@ from . import claw
 
 CANDIDATES = [(32, 32, 1, 256), (32, 32, 1, 512), (32, 32, 0, 256), (32, 32, 0, 512),
               (32, 16, 1, 256), (32, 16, 2, 256), (16, 16, 1, 128)]
+CANDIDATES_UNIFORM = CANDIDATES + [(32, 32, 2, 256), (32, 16, 1, 352), (32, 16, 0, 352), (16, 16, 1, 192),
+                                   (16, 16, 0, 192)]
 CANDIDATES_SWE = [(16, 16, 1, 256), (16, 16, 0, 256), (32, 16, 1, 512), (32, 16, 0, 512)]
 
 
 def candidates_for(H):
     """the tilings the level-step of H's system supports"""
-    return CANDIDATES_SWE if getattr(H, "system", 0) == claw.CLAW_SYS_SHALLOW_WATER else CANDIDATES
+    if getattr(H, "system", 0) == claw.CLAW_SYS_SHALLOW_WATER:
+        return CANDIDATES_SWE
+    return CANDIDATES if H.medium else CANDIDATES_UNIFORM
+
+
 CACHE = os.path.join(os.path.dirname(os.path.abspath(__file__)), "_tune_cache.json")
 _lock = threading.Lock()
 
