@@ -311,6 +311,24 @@ int claw_pack_interiors(claw_ctx* ctx, int32_t level, int32_t box_begin, int32_t
 int claw_unpack_interiors(claw_ctx* ctx, int32_t level, int32_t box_begin, int32_t box_end,
                           const double* packed, double* q, void* stream);
 
+/* `nsteps` coarse steps of a one-level problem (level 0, one run) whose state lives in host memory
+ * (page-locked, for the copies to overlap): every step copies the state from one of host_a, host_b
+ * (the first from host_a), advances it from one of the pools q0, q1 (the first: from q0) into the
+ * other with pulled ghosts, applies Eq. cfl to dt, and copies the new state into the other host
+ * buffer.  The host buffers hold the level's pool, or, with the device buffers stage_in and stage_out
+ * of claw_packed_size doubles (else both NULL), its packed interiors.  The level is taken in npieces
+ * pieces: piece k is the boxes [piece_boxes[k], piece_boxes[k + 1]), the elements [ranges[2 k],
+ * ranges[2 k + 1]) of a host buffer, and is stepped once the pieces needs[need_start[k] ..
+ * need_start[k + 1]) (those holding its boxes and the cells its ghosts come from) have arrived.  Copies
+ * and steps run on streams of the context beside `stream`, which they start from and are joined to;
+ * no buffer may be reused before `stream` has passed that point.  Calls on one context share those
+ * streams.  Errors: CLAW_EINVAL, CLAW_ENOMEM, CLAW_ECUDA. */
+int claw_steps_from_host(claw_ctx* ctx, double* q0, double* q1, const double* aux, double* dt, double* smax,
+                         double* host_a, double* host_b, double* stage_in, double* stage_out,
+                         int32_t nsteps, int32_t npieces, const int32_t* piece_boxes,
+                         const int64_t* ranges, const int32_t* need_start, const int32_t* needs,
+                         void* stream);
+
 /* The same step with one kernel launch per box (the per-patch launch pattern of Sec. 3.1.2,
  * kept as the comparison baseline of the fused launch). */
 int claw_level_step_patchwise(claw_ctx* ctx, int32_t level, const double* q_old, double* q_new,

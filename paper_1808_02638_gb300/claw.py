@@ -91,6 +91,7 @@ _SIGNATURES = {
     "claw_packed_size": ([VP, I32], ctypes.c_longlong),
     "claw_pack_interiors": ([VP, I32, I32, I32, VP, VP, VP], ctypes.c_int),
     "claw_unpack_interiors": ([VP, I32, I32, I32, VP, VP, VP], ctypes.c_int),
+    "claw_steps_from_host": ([VP] * 10 + [I32, I32] + [VP] * 5, ctypes.c_int),
     "claw_level_step_noalloc": ([I32, I32, DBL, DBL, I32, I32, I32, DBL, DBL, VP, VP, VP, VP, VP, VP],
                                 ctypes.c_int),
     "claw_average_down": ([VP, I32, VP, VP, VP], ctypes.c_int),
@@ -137,6 +138,13 @@ def _ptr(t):
         return t
     if not t.is_cuda:
         raise ValueError("libclaw takes device tensors")
+    return t.data_ptr()
+
+
+def _host(t):
+    """host pointer of a contiguous double tensor"""
+    if t.is_cuda:
+        raise ValueError("a host tensor is wanted")
     return t.data_ptr()
 
 
@@ -368,6 +376,21 @@ def claw_pack_interiors(ctx, level, box_begin, box_end, q, packed, stream=None):
 def claw_unpack_interiors(ctx, level, box_begin, box_end, packed, q, stream=None):
     _check("claw_unpack_interiors", load().claw_unpack_interiors(ctx, level, int(box_begin), int(box_end),
                                                                  _ptr(packed), _ptr(q), _stream(stream)))
+
+
+def claw_steps_from_host(ctx, q0, q1, aux, dt, smax, host_a, host_b, stage_in, stage_out, nsteps, pieces, ranges,
+                         needs, stream=None):
+    """pieces: [(first box, end box)], contiguous; ranges: [(begin, end)] elements of a host buffer;
+    needs: [[pieces]]"""
+    import numpy as np
+    boxes = np.array([a for a, _ in pieces] + [pieces[-1][1]], dtype=np.int32)
+    rng = np.array(ranges, dtype=np.int64).reshape(-1)
+    start = np.cumsum([0] + [len(n) for n in needs]).astype(np.int32)
+    flat = np.array([m for n in needs for m in n], dtype=np.int32)
+    _check("claw_steps_from_host", load().claw_steps_from_host(
+        ctx, _ptr(q0), _ptr(q1), _ptr(aux), _ptr(dt), _ptr(smax), _host(host_a), _host(host_b), _ptr(stage_in),
+        _ptr(stage_out), int(nsteps), len(pieces), boxes.ctypes.data, rng.ctypes.data, start.ctypes.data,
+        flat.ctypes.data, _stream(stream)))
 
 
 def claw_level_advance_boxes(ctx, level, box_begin, box_end, q_old, q_new, aux, dt, smax, flags, stream=None):

@@ -125,6 +125,9 @@ void claw_destroy(claw_ctx* ctx)
             free_arena(ctx->lev[L].coeftab);
         }
         free_arena(ctx->scratch);
+        for (cudaStream_t s : ctx->hostloop.streams)
+            if (s) cudaStreamDestroy(s);
+        for (cudaEvent_t e : ctx->hostloop.events) cudaEventDestroy(e);
         cudaFree(ctx->xgrid);
         cudaFree(ctx->err);
         cudaFree(ctx->done);

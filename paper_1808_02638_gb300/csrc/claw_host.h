@@ -101,6 +101,13 @@ struct Locator {
     }
 };
 
+// streams (copies in, copies out, unpack, pack) and events of a context's host-resident loop
+struct HostLoop {
+    static constexpr int kinds = 5;
+    cudaStream_t streams[4] = {};
+    std::vector<cudaEvent_t> events;
+};
+
 struct claw_ctx {
     int device = 0;
     int nsm = 0;
@@ -133,6 +140,7 @@ struct claw_ctx {
     int* xgrid = nullptr;      // the index grids of a regrid transfer (fine then coarse), grown on use
     size_t xgrid_cap = 0;      // ints
     unsigned wait_polls = kWaitPolls;   // first-wait bound of the staged step kernels
+    HostLoop hostloop;
 };
 
 namespace claw_host {

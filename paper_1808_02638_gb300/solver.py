@@ -405,19 +405,32 @@ class Hierarchy:
         the next step reads that one.  The level is taken in `bands` pieces of boxes
         (claw_level_advance_boxes with pulled ghosts): a piece is stepped as soon as it and the
         pieces its ghosts come from have arrived, and copied back as soon as it is stepped, so
-        that the copies in both directions overlap each other and the steps.  Packed pieces are
-        unpacked into the pool and packed out of it on the copy streams.  Eq. cfl follows the
-        last piece of a step.  Measured on the 2048^2 workload: packed state in eight pieces
-        0.71 ms per step (the default), pool state in four pieces 0.80 ms.  Returns the host
-        buffer holding the final state."""
+        that the copies in both directions overlap each other and the steps (one call of the
+        library enqueues it all).  Packed pieces are unpacked into the pool and packed out of it on
+        streams of their own.  Eq. cfl follows the last piece of a step.  bands None: four
+        pieces, one below 3 MB of host buffer.  Measured, us a step of a packed state of 1.6 MB (256^2):
+        66 in one piece, 71 in four; 6.3 MB: 127, 114 and 157 in eight; 25 MB: 359, 221, 236; 101 MB
+        (2048^2): 1316, 676, 704 (a piece costs the host 13 us, a step in one piece overlaps
+        nothing).  Returns the host buffer holding the final state."""
         if self.nlev != 1 or self.nruns != 1:
             raise ValueError("host-resident stepping is for one-level hierarchies of one run")
+        plain = all(t.dtype == torch.float64 and t.is_contiguous() for t in (host_a, host_b))
+        if not plain:   # other types and strides go through plain buffers
+            a, b = (torch.empty(host_a.numel(), dtype=torch.float64).pin_memory() for _ in range(2))
+            a.copy_(host_a)
+            out = self.steps_from_host(a, b, nsteps, bands)
+            torch.cuda.current_stream(self.dev).synchronize()
+            host_a.copy_(a)
+            if nsteps:
+                host_b.copy_(b)
+            return host_a if out is a else host_b
         packed = host_a.numel() == self.packed_size(0)
         if bands is None:
-            bands = 8 if packed else 4
+            bands = 4 if host_a.numel() * 8 >= 3 << 20 else 1
         if not hasattr(self, "_band_cache") or self._band_cache[0] != bands:
             self._band_cache = (bands, self._bands(bands))
         parts, ranges, needs = self._band_cache[1]
+        stage = (None, None)
         if packed:
             b = self.boxes[0]
             offs = np.concatenate([[0], np.cumsum(3 * b.nx.astype(np.int64) * b.ny)])
@@ -425,74 +438,21 @@ class Hierarchy:
             if getattr(self, "_stage", None) is None or self._stage[0].numel() != host_a.numel():
                 self._stage = (torch.empty(host_a.numel(), dtype=torch.float64, device=self.dev),
                                torch.empty(host_a.numel(), dtype=torch.float64, device=self.dev))
-            st_in, st_out = self._stage
+            stage = self._stage
         elif host_a.numel() != self.q[0][0].numel():
             raise ValueError("host buffers must hold the level's pool or its packed interiors")
-        comp = torch.cuda.current_stream(self.dev)
-        s_in, s_out = torch.cuda.Stream(device=self.dev), torch.cuda.Stream(device=self.dev)
-        # packed form: the unpack and pack kernels run on their own streams, so that the copy
-        # streams carry copies only
-        s_un, s_pk = torch.cuda.Stream(device=self.dev), torch.cuda.Stream(device=self.dev)
-        arrived = [torch.cuda.Event() for _ in parts]
-        stepped = [torch.cuda.Event() for _ in parts]
-        landed = [torch.cuda.Event() for _ in parts]      # a packed piece is in the staging buffer
-        unpacked = [None] * len(parts)                    # ... and has been unpacked from it
-        packed_ev = [torch.cuda.Event() for _ in parts]   # a piece is packed into the out staging
-        left = [None] * len(parts)
-        src, dst = host_a, host_b
-        for st in (s_in, s_out, s_un, s_pk):
-            st.wait_stream(comp)
-        flags = claw.CLAW_ADVANCE_PULL_GHOSTS
-        for _ in range(nsteps):
-            q, qn = self.q[0][self.cur[0]], self.q[0][1 - self.cur[0]]
-            for k, (a, b) in enumerate(ranges):
-                if left[k] is not None:
-                    s_in.wait_event(left[k])   # this piece of the previous step is back on the host
-                if packed:
-                    if unpacked[k] is not None:
-                        s_in.wait_event(unpacked[k])   # its staging slot has been read
-                    with torch.cuda.stream(s_in):
-                        st_in[a:b].copy_(src[a:b], non_blocking=True)
-                    landed[k].record(s_in)
-                    s_un.wait_event(landed[k])
-                    claw.claw_unpack_interiors(self.ctx, 0, parts[k][0], parts[k][1], st_in, q, s_un)
-                    ev = torch.cuda.Event()
-                    ev.record(s_un)
-                    unpacked[k] = ev
-                    arrived[k] = ev
-                else:
-                    with torch.cuda.stream(s_in):
-                        q[a:b].copy_(src[a:b], non_blocking=True)
-                    arrived[k].record(s_in)
-            for k, (b0, b1) in enumerate(parts):
-                for m in needs[k]:
-                    comp.wait_event(arrived[m])
-                claw.claw_level_advance_boxes(self.ctx, 0, b0, b1, q, qn, self.aux[0], self.dt, self.smax, flags,
-                                              comp)
-                stepped[k].record(comp)
-            claw.claw_dt_update(self.ctx, 0, self.smax, self.dt, comp)
-            for k, (a, b) in enumerate(ranges):
-                if packed:
-                    s_pk.wait_event(stepped[k])
-                    if left[k] is not None:
-                        s_pk.wait_event(left[k])   # its out staging slot has been copied out
-                    claw.claw_pack_interiors(self.ctx, 0, parts[k][0], parts[k][1], qn, st_out, s_pk)
-                    packed_ev[k].record(s_pk)
-                    s_out.wait_event(packed_ev[k])
-                    with torch.cuda.stream(s_out):
-                        dst[a:b].copy_(st_out[a:b], non_blocking=True)
-                else:
-                    s_out.wait_event(stepped[k])
-                    with torch.cuda.stream(s_out):
-                        dst[a:b].copy_(qn[a:b], non_blocking=True)
-                ev = torch.cuda.Event()
-                ev.record(s_out)
-                left[k] = ev
-            self.cur[0] ^= 1
-            src, dst = dst, src
-        for st in (s_out, s_in, s_un, s_pk):
-            comp.wait_stream(st)
-        return src
+        if host_b.numel() != host_a.numel():
+            raise ValueError("host buffers must have the same length")
+        c = self.cur[0]
+        with torch.cuda.device(self.dev):
+            claw.claw_steps_from_host(self.ctx, self.q[0][c], self.q[0][1 - c], self.aux[0], self.dt, self.smax,
+                                      host_a, host_b, *stage, nsteps, parts, ranges, needs)
+            # torch's allocators learn that the buffers are in use up to here on this stream
+            for t in (host_a, host_b):
+                if t.is_pinned():
+                    torch.empty(1, dtype=torch.float64, device=self.dev).copy_(t.view(-1)[:1], non_blocking=True)
+        self.cur[0] ^= nsteps & 1
+        return host_b if nsteps & 1 else host_a
 
     def launches_per_coarse_step(self):
         """kernels one coarse step enqueues (counted from the library's own counter)."""
