@@ -10,8 +10,8 @@
 // fused multiply-add per component).
 //
 // Precision: with e the smallest exponent such that |du|, |dv|, |dp| / Z < 2^e on every edge of the
-// tile, the unit is 2^(e - 58).  Sums and limiters are exact, a product errs by less than a unit and
-// a half, and the increment of a cell by a few units: about 2^-56 of the tile's largest jump, where
+// tile, the unit is 2^(e - 58).  Sums and limiters are exact, a product errs by less than 2.5
+// units, and the increment of a cell by a few units: about 2^-56 of the tile's largest jump, where
 // a double's rounding is 2^-53 of the value at hand.  A tile is stepped this way only if at every
 // edge the state next to it or the jump across it is at least 2^(e - 4): the error then is below
 // the rounding of the local state.  Every other tile (a state on a zero background in front of a
@@ -38,13 +38,13 @@ __device__ __forceinline__ Coef coef_bits(long long c)   // c 2^64, at most 2^62
     return r;
 }
 
-// v c to within a unit and a half: of the two cross products only the upper words are formed
-// (each rounded down, the 1 makes up for the mean of the two), the product of the low words,
-// below half a unit, is dropped
+// v c from 2.5 units below to half a unit above: of the two cross products only the upper words are
+// formed (each rounded down) and the product of the low words, below half a unit, is dropped.  0 gives
+// 0: where nothing changes, nothing may.
 __device__ __forceinline__ long long mul(long long v, Coef c)
 {
     const int vh = (int)(v >> 32);
-    const int t = __mulhi(vh, c.lo) + 1 + (int)__umulhi((unsigned)v, (unsigned)c.hi);   // |.| <= 2^30 each
+    const int t = __mulhi(vh, c.lo) + (int)__umulhi((unsigned)v, (unsigned)c.hi);   // |.| <= 2^30 each
     return (long long)vh * c.hi + t;
 }
 

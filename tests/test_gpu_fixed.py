@@ -155,3 +155,33 @@ def _long_step(q, lam):
     return np.stack([q[0, i, i] - lam * (xp[i] + yp[:, i] + np.diff(fp, axis=1) + np.diff(gp, axis=0)),
                      q[1, i, i] - lam * (xu[i] + np.diff(fu, axis=1)),
                      q[2, i, i] - lam * (yv[:, i] + np.diff(gv, axis=0))])
+
+
+@pytest.mark.parametrize("medium", [False, True])
+@pytest.mark.parametrize("limiter", [0, 1, 2, 3, 4])
+def test_cells_out_of_a_disturbance_s_reach_do_not_change(limiter, medium):
+    # one disturbed cell in a state of rest on a large pressure: q_new is q bit for bit outside the
+    # stencil (two cells in each direction), and zero velocities stay exactly zero there
+    n = 40
+    run = inputs.Run(0.0, 0.0, 1.0, 1.0, limiter=limiter)
+    run.levels = [inputs.Level(n, n, 1.0 / n, 1.0 / n, [(0, 0, n, n)])]
+    pool = np.zeros(run.levels[0].qsize)
+    q = inputs.box_view(pool, 0, n, n, 3)
+    q[0] = 1.0
+    q[0, 22, 17] = 1.25
+    q[1, 22, 17] = 0.125
+    kw = dict(rho0=1.0, K0=4.0)
+    args = []
+    if medium:
+        args = [[[inputs.coef_pool(run.levels[0], f, 1)]] for f in
+                (inputs.smooth_field(1, n, n, 0.5, 2.0), inputs.smooth_field(2, n, n, 1.0, 8.0))]
+        kw = {}
+    H = Hierarchy([run], [[pool]], *args, **kw)
+    H.init_dt()
+    claw.claw_level_step(H.ctx, 0, H.q[0][0], H.q[0][1], H.aux[0], H.dt, H.smax)
+    new = H.interior(0, 0, 0, pool=H.q[0][1])
+    old = q[:, 2:-2, 2:-2]
+    far = np.ones((n, n), dtype=bool)
+    far[18:23, 13:18] = False
+    assert np.array_equal(new[:, far], old[:, far]) and not np.array_equal(new, old)
+    assert H.sync_status() == claw.CLAW_OK
