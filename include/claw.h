@@ -469,6 +469,17 @@ int claw_reflux_fine(claw_ctx* ctx, int32_t fine_level, const double* q_f, const
  * summed per cell in table order (deterministic) */
 int claw_reflux_apply(claw_ctx* ctx, int32_t fine_level, const double* buf, const double* dt,
                       double* q_c_new, void* stream);
+/* claw_level_step on level `level` (ghosts of q_old filled) whose launch also evaluates, on CTAs beside
+ * those that step, the fine part at the level's interface with the coarser one (buf_fine, from q_old and
+ * the coarser level's state qc_old at its step's start; NULL: none) and the coarse part at its interface
+ * with the finer level (buf_coarse, from q_old; NULL: none): claw_reflux_fine, claw_reflux_coarse and
+ * claw_level_step in one launch, with the same results.  Errors as theirs. */
+int claw_level_step_reflux(claw_ctx* ctx, int32_t level, const double* q_old, double* q_new, const double* dt,
+                           double* smax, const double* qc_old, double* buf_fine, double* buf_coarse,
+                           void* stream);
+/* claw_average_down and claw_reflux_apply in one launch, with the same results */
+int claw_average_down_reflux(claw_ctx* ctx, int32_t fine_level, const double* q_f, double* q_c_new,
+                             const double* buf, const double* dt, void* stream);
 
 /* ---- Regridding (Sec. 2.2: every K steps the finer levels are regenerated from flagged cells
  * clustered with the algorithm of Berger and Rigoutsos; Sec. 4.3: cutoff and regrid interval).

@@ -73,6 +73,8 @@ _SIGNATURES = {
     "claw_reflux_coarse": ([VP, I32, VP, VP, VP, VP], ctypes.c_int),
     "claw_reflux_fine": ([VP, I32, VP, VP, VP, VP, VP], ctypes.c_int),
     "claw_reflux_apply": ([VP, I32, VP, VP, VP, VP], ctypes.c_int),
+    "claw_level_step_reflux": ([VP, I32] + [VP] * 8, ctypes.c_int),
+    "claw_average_down_reflux": ([VP, I32] + [VP] * 5, ctypes.c_int),
     "claw_fill_ghost": ([VP, I32, VP, VP, VP, DBL, VP], ctypes.c_int),
     "claw_fill_ghost_adjoint": ([VP, I32, VP, VP, VP, VP, VP, DBL, VP], ctypes.c_int),
     "claw_fill_ghost_interp_adjoint": ([VP, I32, VP, VP, VP, VP, VP, DBL, VP], ctypes.c_int),
@@ -300,6 +302,17 @@ def claw_reflux_fine(ctx, fine_level, q_f, q_c_old, dt, buf, stream=None):
 def claw_reflux_apply(ctx, fine_level, buf, dt, q_c_new, stream=None):
     _check("claw_reflux_apply", load().claw_reflux_apply(ctx, fine_level, _ptr(buf), _ptr(dt), _ptr(q_c_new),
                                                          _stream(stream)))
+
+
+def claw_level_step_reflux(ctx, level, q_old, q_new, dt, smax, qc_old, buf_fine, buf_coarse, stream=None):
+    _check("claw_level_step_reflux", load().claw_level_step_reflux(
+        ctx, level, _ptr(q_old), _ptr(q_new), _ptr(dt), _ptr(smax), _ptr(qc_old), _ptr(buf_fine), _ptr(buf_coarse),
+        _stream(stream)))
+
+
+def claw_average_down_reflux(ctx, fine_level, qf, q_c_new, buf, dt, stream=None):
+    _check("claw_average_down_reflux", load().claw_average_down_reflux(
+        ctx, fine_level, _ptr(qf), _ptr(q_c_new), _ptr(buf), _ptr(dt), _stream(stream)))
 
 
 def claw_medium_aux_adjoint(ctx, level, rho, K, g_aux, g_rho, g_K, stream=None):

@@ -284,6 +284,8 @@ int claw_set_level(claw_ctx* ctx, int32_t L, const claw_box* boxes, int32_t nbox
     d.ncopy = (int)gt.nrects;
     d.ninterp = (int)gt.ncells;
     d.navg = (int)avg.size();
+    d.avg_cells = 0;
+    for (const AvgRect& r : avg) d.avg_cells = std::max(d.avg_cells, r.w * r.h);
     // a cell-wise medium fills its coefficient pools' ghosts: those tables are built now, a
     // uniform medium builds them on first use
     if (ctx->medium && (rc = build_coef_tables(ctx, L))) return rc;
@@ -377,13 +379,9 @@ int claw_fill_ghost(claw_ctx* ctx, int32_t L, double* q, const double* qc_old, c
     if (d.ninterp > 0 && (!qc_old || !qc_new || !(tau >= 0.0 && tau <= 1.0))) return CLAW_EINVAL;
     DevGuard g(ctx->device);
     cudaStream_t s = (cudaStream_t)stream;
-    cudaError_t e = d.ncopy ? launch_fill_copy(d.copies, d.copy_start, d.ncopy_blocks, q, s) : cudaSuccess;
-    ctx->launches += d.ncopy > 0;
-    if (e == cudaSuccess) {
-        e = launch_fill_interp(d.interps, d.ninterp, q, qc_old, qc_new, tau, s);
-        ctx->launches += d.ninterp > 0;
-    }
-    return cuda_rc(e);
+    ctx->launches += d.ncopy > 0 || d.ninterp > 0;
+    return cuda_rc(launch_fill_ghost(d.copies, d.copy_start, d.ncopy ? d.ncopy_blocks : 0, d.interps, d.ninterp, q,
+                                     qc_old, qc_new, tau, s));
 }
 
 int claw_fill_ghost_interp(claw_ctx* ctx, int32_t L, double* q, const double* qc_old, const double* qc_new,
@@ -703,7 +701,7 @@ int claw_average_down(claw_ctx* ctx, int32_t fl, const double* qf, double* qc, v
     DevGuard g(ctx->device);
     const LevelDev& d = ctx->lev[fl];
     ctx->launches += d.navg > 0;
-    return cuda_rc(launch_average(d.avgs, d.navg, d.ratio, qf, qc, (cudaStream_t)stream));
+    return cuda_rc(launch_average(d.avgs, d.navg, d.avg_cells, d.ratio, qf, qc, (cudaStream_t)stream));
 }
 
 int claw_average_down_adjoint(claw_ctx* ctx, int32_t fl, double* lf, double* lc, void* stream)
@@ -826,17 +824,38 @@ int claw_reflux_buffer_size(claw_ctx* ctx, int32_t L)
     return rc ? -rc : 3 * ctx->lev[L].nreflux * (1 + ctx->lev[L].ratio);
 }
 
+// the coarse (fine = 0) or fine part of the fix at the interface of levels L - 1 and L
+static RefluxJob reflux_job(const claw_ctx* ctx, int L, int fine, const double* qf, const double* qc, double* buf)
+{
+    const LevelDev& d = ctx->lev[L];
+    RefluxJob J;
+    J.recs = d.reflux;
+    J.n = d.nreflux;
+    J.cp = ctx->lev[L - 1].patches;
+    J.fp = d.patches;
+    J.qf = qf;
+    J.qc = qc;
+    J.buf = buf;
+    J.ratio = d.ratio;
+    J.fine = fine;
+    return J;
+}
+
+static int launch_reflux_job(claw_ctx* ctx, int L, const RefluxJob& job, const double* dt, void* stream)
+{
+    DevGuard g(ctx->device);
+    StepArgs k = make_args(ctx, L, nullptr, nullptr, nullptr, dt, nullptr);
+    k.reflux[k.nreflux++] = job;
+    ctx->launches += job.n > 0;
+    return cuda_rc(launch_reflux(k, ctx->limiter, (cudaStream_t)stream));
+}
+
 int claw_reflux_coarse(claw_ctx* ctx, int32_t L, const double* q_c_old, const double* dt, double* buf, void* stream)
 {
     int rc = reflux_check(ctx, L);
     if (rc) return rc;
     if (!q_c_old || !dt || !buf) return CLAW_EINVAL;
-    DevGuard g(ctx->device);
-    const LevelDev& d = ctx->lev[L];
-    const StepArgs k = make_args(ctx, L - 1, nullptr, nullptr, nullptr, dt, nullptr);
-    ctx->launches += d.nreflux > 0;
-    return cuda_rc(launch_reflux_coarse(d.reflux, d.nreflux, ctx->lev[L - 1].patches, q_c_old, dt, buf, d.ratio, k,
-                                        ctx->limiter, (cudaStream_t)stream));
+    return launch_reflux_job(ctx, L - 1, reflux_job(ctx, L, 0, nullptr, q_c_old, buf), dt, stream);
 }
 
 int claw_reflux_fine(claw_ctx* ctx, int32_t L, const double* q_f, const double* q_c_old, const double* dt, double* buf,
@@ -845,12 +864,51 @@ int claw_reflux_fine(claw_ctx* ctx, int32_t L, const double* q_f, const double* 
     int rc = reflux_check(ctx, L);
     if (rc) return rc;
     if (!q_f || !q_c_old || !dt || !buf) return CLAW_EINVAL;
+    return launch_reflux_job(ctx, L, reflux_job(ctx, L, 1, q_f, q_c_old, buf), dt, stream);
+}
+
+int claw_level_step_reflux(claw_ctx* ctx, int32_t L, const double* q_old, double* q_new, const double* dt,
+                           double* smax, const double* qc_old, double* buf_fine, double* buf_coarse, void* stream)
+{
+    int rc = check_step_args(ctx, L, q_old, q_new, nullptr, dt, smax);
+    if (rc) return rc;
+    if (ctx->medium != 0 || (buf_fine && (L < 1 || !qc_old || qc_old == q_new)) ||
+        (buf_coarse && (L + 1 >= CLAW_MAXLEV || !ctx->set[L + 1])))
+        return CLAW_EINVAL;
+    DevGuard g(ctx->device);
+    LevelDev& d = ctx->lev[L];
+    cudaStream_t s = (cudaStream_t)stream;
+    StepArgs a = make_args(ctx, L, q_old, q_new, nullptr, dt, smax);
+    if (buf_fine) a.reflux[a.nreflux++] = reflux_job(ctx, L, 1, q_old, qc_old, buf_fine);
+    if (buf_coarse) a.reflux[a.nreflux++] = reflux_job(ctx, L + 1, 0, nullptr, q_old, buf_coarse);
+    if (d.ntiles == 0) {
+        ctx->launches += a.nreflux > 0;
+        return cuda_rc(launch_reflux(a, ctx->limiter, s));
+    }
+    int staging = d.staging;
+    if (staging >= 1) {
+        a.tmaps = get_tmaps(ctx, L, q_old, s);
+        if (!a.tmaps) staging = 0;
+    }
+    const int per_sm = step_max_ctas_per_sm(ctx->kind(), ctx->limiter, d.tx, d.ty, d.nt, staging, false, false, false,
+                                            a.tcum != nullptr);
+    if (per_sm <= 0) return CLAW_ECUDA;
+    const int grid = std::min(d.ntiles, per_sm * ctx->nsm);
+    ctx->launches += 1;
+    return cuda_rc(launch_step(a, ctx->kind(), ctx->limiter, d.tx, d.ty, d.nt, staging, grid, s,
+                               std::max(per_sm * ctx->nsm - grid, ctx->nsm)));
+}
+
+static int average_reflux(claw_ctx* ctx, int L, const double* qf, const double* buf, const double* dt, double* qc,
+                          void* stream)
+{
     DevGuard g(ctx->device);
     const LevelDev& d = ctx->lev[L];
-    const StepArgs k = make_args(ctx, L, nullptr, nullptr, nullptr, dt, nullptr);
-    ctx->launches += d.nreflux > 0;
-    return cuda_rc(launch_reflux_fine(d.reflux, d.nreflux, ctx->lev[L - 1].patches, d.patches, q_f, q_c_old, dt, buf,
-                                      d.ratio, k, ctx->limiter, (cudaStream_t)stream));
+    const int navg = qf ? d.navg : 0;
+    ctx->launches += navg > 0 || d.nreflux_groups > 0;
+    return cuda_rc(launch_average_reflux(d.avgs, navg, d.avg_cells, qf, d.reflux, d.nreflux, d.reflux_group,
+                                         d.nreflux_groups, d.ratio, ctx->lev[L - 1].patches, dt, buf, qc,
+                                         (cudaStream_t)stream));
 }
 
 int claw_reflux_apply(claw_ctx* ctx, int32_t L, const double* buf, const double* dt, double* q_c_new, void* stream)
@@ -858,11 +916,16 @@ int claw_reflux_apply(claw_ctx* ctx, int32_t L, const double* buf, const double*
     int rc = reflux_check(ctx, L);
     if (rc) return rc;
     if (!buf || !dt || !q_c_new) return CLAW_EINVAL;
-    DevGuard g(ctx->device);
-    const LevelDev& d = ctx->lev[L];
-    ctx->launches += d.nreflux_groups > 0;
-    return cuda_rc(launch_reflux_apply(d.reflux, d.nreflux, d.reflux_group, d.nreflux_groups, d.ratio,
-                                       ctx->lev[L - 1].patches, dt, buf, q_c_new, (cudaStream_t)stream));
+    return average_reflux(ctx, L, nullptr, buf, dt, q_c_new, stream);
+}
+
+int claw_average_down_reflux(claw_ctx* ctx, int32_t L, const double* qf, double* q_c_new, const double* buf,
+                             const double* dt, void* stream)
+{
+    int rc = reflux_check(ctx, L);
+    if (rc) return rc;
+    if (!qf || !buf || !dt || !q_c_new) return CLAW_EINVAL;
+    return average_reflux(ctx, L, qf, buf, dt, q_c_new, stream);
 }
 
 int claw_sync_status(claw_ctx* ctx)

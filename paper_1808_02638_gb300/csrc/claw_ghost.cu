@@ -5,6 +5,7 @@
 // (claw_set_level) so that each launch is a flat loop over tasks.
 #include <cuda_runtime.h>
 
+#include "claw_average.cuh"
 #include "claw_interp.cuh"
 
 namespace claw {
@@ -68,9 +69,8 @@ __device__ __forceinline__ bool negated(int flags, int m)
     return (m == 1 && (flags & 1)) || (m == 2 && (flags & 2));
 }
 
-__global__ void __launch_bounds__(kCopyThreads) fill_copy_kernel(const CopyRect* __restrict__ rects,
-                                                                 const int* __restrict__ start,
-                                                                 double* __restrict__ q, int ncomp)
+__device__ __forceinline__ void copy_block(const CopyRect* __restrict__ rects, const int* __restrict__ start,
+                                           double* __restrict__ q, int ncomp)
 {
     __shared__ CopyChunk c;
     const int r_lo = start[blockIdx.x], r_hi = start[blockIdx.x + 1];
@@ -98,6 +98,13 @@ __global__ void __launch_bounds__(kCopyThreads) fill_copy_kernel(const CopyRect*
         }
         __syncthreads();   // the chunk is restaged
     }
+}
+
+__global__ void __launch_bounds__(kCopyThreads) fill_copy_kernel(const CopyRect* __restrict__ rects,
+                                                                 const int* __restrict__ start,
+                                                                 double* __restrict__ q, int ncomp)
+{
+    copy_block(rects, start, q, ncomp);
 }
 
 // reverse: ghost adjoint flows into its source, then the ghost adjoint is cleared.  Sources
@@ -154,6 +161,26 @@ __global__ void fill_interp_kernel(const InterpCell* __restrict__ cells, int n, 
     q[C.dst + m * C.dplane] = interp_value(C, m, cold, cnew, tau);
 }
 
+// both kinds of ghosts in one launch (they are disjoint, and neither reads the other): blocks
+// [0, ncopy) copy, the others interpolate, a thread per (cell, component).  As two launches one after
+// the other a fill of a small level took 9.5 us.
+__global__ void __launch_bounds__(kCopyThreads) fill_ghost_kernel(const CopyRect* __restrict__ rects,
+                                                                  const int* __restrict__ start, int ncopy,
+                                                                  const InterpCell* __restrict__ cells, int n,
+                                                                  double* q, const double* __restrict__ cold,
+                                                                  const double* __restrict__ cnew, double tau)
+{
+    if ((int)blockIdx.x < ncopy) {
+        copy_block(rects, start, q, 3);
+        return;
+    }
+    const int k = ((int)blockIdx.x - ncopy) * kCopyThreads + (int)threadIdx.x;
+    if (k >= 3 * n) return;
+    const int i = k / 3, m = k - 3 * i;
+    const InterpCell C = cells[i];
+    q[C.dst + m * C.dplane] = interp_value(C, m, cold, cnew, tau);
+}
+
 __global__ void fill_interp_adjoint_kernel(const InterpCell* __restrict__ cells, int n,
                                            double* __restrict__ lam, double* __restrict__ lco,
                                            double* __restrict__ lcn, const double* __restrict__ cold,
@@ -199,6 +226,15 @@ cudaError_t launch_fill_interp(const InterpCell* c, int n, double* q, const doub
     return cudaGetLastError();
 }
 
+cudaError_t launch_fill_ghost(const CopyRect* r, const int* start, int nblocks, const InterpCell* c, int n, double* q,
+                              const double* cold, const double* cnew, double tau, cudaStream_t s)
+{
+    const int blocks = std::max(nblocks, 0) + div_up(3LL * std::max(n, 0), kCopyThreads);
+    if (blocks == 0) return cudaSuccess;
+    fill_ghost_kernel<<<blocks, kCopyThreads, 0, s>>>(r, start, std::max(nblocks, 0), c, n, q, cold, cnew, tau);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_fill_interp_adjoint(const InterpCell* c, int n, double* lam, double* lco,
                                        double* lcn, const double* cold, const double* cnew,
                                        double tau, cudaStream_t s)
@@ -209,23 +245,11 @@ cudaError_t launch_fill_interp_adjoint(const InterpCell* c, int n, double* lam, 
 }
 
 // ------------------------------------------------------------------------ averaging
-// block per rectangle, thread per (coarse cell, component); the r x r children are summed
-// row by row and divided by r^2
-__global__ void average_kernel(const AvgRect* __restrict__ rects, int ratio, const double* __restrict__ qf,
-                               double* __restrict__ qc)
+__global__ void __launch_bounds__(kAverageThreads) average_kernel(const AvgRect* __restrict__ rects, int nrects, int ratio,
+                                                                  const double* __restrict__ qf,
+                                                                  double* __restrict__ qc)
 {
-    const AvgRect R = rects[blockIdx.x];
-    const int cells = R.w * R.h;
-    const double rr = (double)(ratio * ratio);
-    for (int k = threadIdx.x; k < 3 * cells; k += blockDim.x) {
-        const int m = k / cells, e = k - m * cells;
-        const int y = e / R.w, x = e - y * R.w;
-        const double* f = qf + R.fsrc + m * R.fplane + (long long)y * ratio * R.fpitch + (long long)x * ratio;
-        double s = 0.0;
-        for (int b = 0; b < ratio; ++b)
-            for (int a = 0; a < ratio; ++a) s += f[(long long)b * R.fpitch + a];
-        qc[R.cdst + m * R.cplane + (long long)y * R.cpitch + x] = s / rr;
-    }
+    average_block(rects, nrects, gridDim.x, ratio, qf, qc);
 }
 
 __global__ void average_adjoint_kernel(const AvgRect* __restrict__ rects, int ratio, double* __restrict__ lf,
@@ -246,10 +270,11 @@ __global__ void average_adjoint_kernel(const AvgRect* __restrict__ rects, int ra
     }
 }
 
-cudaError_t launch_average(const AvgRect* r, int n, int ratio, const double* qf, double* qc, cudaStream_t s)
+cudaError_t launch_average(const AvgRect* r, int n, int max_cells, int ratio, const double* qf, double* qc,
+                           cudaStream_t s)
 {
     if (n <= 0) return cudaSuccess;
-    average_kernel<<<n, 256, 0, s>>>(r, ratio, qf, qc);
+    average_kernel<<<average_blocks(n, max_cells), kAverageThreads, 0, s>>>(r, n, ratio, qf, qc);
     return cudaGetLastError();
 }
 

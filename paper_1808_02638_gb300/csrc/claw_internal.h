@@ -143,6 +143,20 @@ struct FillJob {
     double tau = 0.0;
 };
 
+// The coarse or the fine part of the conservation fix at one level's interface (claw_reflux.cuh), run
+// by a launch of its own or by spare CTAs of a level-step launch.
+struct RefluxJob {
+    const RefluxRec* recs = nullptr;
+    int n = 0;
+    const PatchDev* cp = nullptr;   // boxes of the coarse and the fine level
+    const PatchDev* fp = nullptr;
+    const double* qf = nullptr;     // fine: the level's state; qc: the coarse level's state at the coarse step's start
+    const double* qc = nullptr;
+    double* buf = nullptr;
+    int ratio = 1;
+    int fine = 0;
+};
+
 // Coarse cells [0,w) x [0,h) at cdst, each the mean of r x r fine cells at fsrc.
 struct AvgRect {
     long long cdst, fsrc;
@@ -167,6 +181,7 @@ struct LevelDev {
     int ncopy = 0;
     int ninterp = 0;
     int navg = 0;          // averaging rects into the coarser level
+    int avg_cells = 0;     // coarse cells of the largest of them
     int ratio = 1;
     int tx = 32, ty = 32, staging = 1, nt = 0;   // tile, staging, threads per CTA (0: default)
     bool tiling_set = false;   // claw_set_tiling chose tx, ty, staging, nt (kept by claw_set_level)
@@ -243,7 +258,7 @@ struct StepArgs {
     // scheme
     int order = 2, transverse = 2;
     double rho0 = 1.0, K0 = 1.0;   // uniform medium
-    double Z0 = 1.0, c0 = 1.0, iZ = 1.0;   // its impedance, speed and 1 / Z0 (set_medium)
+    double Z0 = 1.0, c0 = 1.0, iZ = 1.0, irho = 1.0;   // its impedance, speed, 1 / Z0, 1 / rho0 (set_medium)
     void set_medium(double rho, double K)
     {
         rho0 = rho;
@@ -251,6 +266,7 @@ struct StepArgs {
         Z0 = std::sqrt(K * rho);
         c0 = std::sqrt(K / rho);
         iZ = 1.0 / Z0;
+        irho = 1.0 / rho;
     }
     double grav = 0.0;             // shallow water
     int swe = 0;                   // 1: the shallow water system (the conservation fix reads it)
@@ -278,6 +294,10 @@ struct StepArgs {
     int step_grid = 0;
     int nfill = 0;
     FillJob fills[2];
+    // CTAs [reflux_grid, gridDim.x) (the last of those beside the stepping ones) run the reflux jobs
+    int reflux_grid = 0;
+    int nreflux = 0;
+    RefluxJob reflux[2];
 };
 
 // error flag bits written by kernels
@@ -315,7 +335,11 @@ cudaError_t launch_fill_copy_adjoint(const CopyRect* r, const int* start, int nb
 cudaError_t launch_fill_interp_adjoint(const InterpCell* c, int n, double* lam, double* lco,
                                        double* lcn, const double* cold, const double* cnew,
                                        double tau, cudaStream_t s);
-cudaError_t launch_average(const AvgRect* r, int n, int ratio, const double* qf, double* qc,
+// both kinds of ghosts of a level in one launch
+cudaError_t launch_fill_ghost(const CopyRect* r, const int* start, int nblocks, const InterpCell* c, int n, double* q,
+                              const double* cold, const double* cnew, double tau, cudaStream_t s);
+// max_cells: the coarse cells of the largest rectangle
+cudaError_t launch_average(const AvgRect* r, int n, int max_cells, int ratio, const double* qf, double* qc,
                            cudaStream_t s);
 cudaError_t launch_average_adjoint(const AvgRect* r, int n, int ratio, double* lf, double* lc,
                                    cudaStream_t s);
@@ -338,16 +362,13 @@ cudaError_t launch_regrid_transfer(const XferBox* nb, int n_new, const XferBox* 
                                    long long ccells, const double* q_old, const double* q_coarse, double* q_new,
                                    int* err, cudaStream_t s);
 
-// conservation fix (uniform medium): buf holds 3 doubles per interface record (the coarse
+// conservation fix (uniform medium, shallow water): buf holds 3 doubles per interface record (the coarse
 // parts) followed by 3 per record and fine edge (the fine parts, summed over the substeps)
-// (k: the scheme's order, transverse mode and uniform medium rho0, K0)
-cudaError_t launch_reflux_coarse(const RefluxRec* rec, int n, const PatchDev* cp, const double* qc, const double* dt,
-                                 double* buf, int ratio, const StepArgs& k, int limiter, cudaStream_t s);
-cudaError_t launch_reflux_fine(const RefluxRec* rec, int n, const PatchDev* cp, const PatchDev* fp, const double* qf,
-                               const double* qc, const double* dt, double* buf, int ratio, const StepArgs& k,
-                               int limiter, cudaStream_t s);
-cudaError_t launch_reflux_apply(const RefluxRec* rec, int n, const int* group, int ngroups, int ratio,
-                                const PatchDev* cp, const double* dt, const double* buf, double* qc, cudaStream_t s);
+cudaError_t launch_reflux(const StepArgs& a, int limiter, cudaStream_t s);   // a.reflux, the scheme and dt
+// the average (nrects may be 0) and the fix's corrections in one launch
+cudaError_t launch_average_reflux(const AvgRect* r, int nrects, int max_cells, const double* qf, const RefluxRec* rec,
+                                  int n, const int* group, int ngroups, int ratio, const PatchDev* cp,
+                                  const double* dt, const double* buf, double* qc, cudaStream_t s);
 cudaError_t launch_cfl_max(const PatchDev* p, int n, int max_rows, int medium, double c0, const double* aux,
                            double* smax, cudaStream_t s);
 cudaError_t launch_pack(const PatchDev* p, const long long* poff, int b0, int b1, int max_rows, double* q,

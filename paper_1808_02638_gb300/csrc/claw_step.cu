@@ -73,12 +73,20 @@ cudaError_t launch_step(const StepArgs& a, int kind, int limiter, int tx, int ty
     if (e != cudaSuccess) return e;
     long long items = 0;   // (ghost cell, component) pairs of the fill jobs
     for (int j = 0; j < a.nfill; ++j) items += 3LL * a.fills[j].n;
+    long long edges = 0;   // of the reflux jobs, eight threads each
+    for (int j = 0; j < a.nreflux; ++j) edges += a.reflux[j].fine ? a.reflux[j].n * (long long)a.reflux[j].ratio : a.reflux[j].n;
+    const int reflux = (int)std::min<long long>((edges * 8 + k.nt - 1) / k.nt, std::max(spare, 1));
     if (items > 0) {
         // one pair per thread where `spare` CTAs allow, else those CTAs stride over them
         StepArgs b = a;
         b.step_grid = grid;
         const int extra = (int)std::min<long long>((items + k.nt - 1) / k.nt, std::max(spare, 1));
-        k.fn<<<grid + extra, k.nt, a.tcum ? k.smem_walk : k.smem, s>>>(b);
+        b.reflux_grid = grid + extra;
+        k.fn<<<grid + extra + reflux, k.nt, a.tcum ? k.smem_walk : k.smem, s>>>(b);
+    } else if (reflux > 0) {
+        StepArgs b = a;
+        b.step_grid = b.reflux_grid = grid;
+        k.fn<<<grid + reflux, k.nt, a.tcum ? k.smem_walk : k.smem, s>>>(b);
     } else {
         k.fn<<<grid, k.nt, a.tcum ? k.smem_walk : k.smem, s>>>(a);
     }

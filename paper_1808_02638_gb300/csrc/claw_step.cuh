@@ -322,7 +322,8 @@ __device__ __forceinline__ void fill_jobs(const StepArgs& A)
 {
     const long long n0 = 3LL * A.fills[0].n;
     const long long n = n0 + (A.nfill > 1 ? 3LL * A.fills[1].n : 0LL);
-    const long long stride = (long long)(gridDim.x - A.step_grid) * NT;
+    const int end = A.nreflux ? A.reflux_grid : (int)gridDim.x;
+    const long long stride = (long long)(end - A.step_grid) * NT;
     for (long long k = (long long)(blockIdx.x - A.step_grid) * NT + threadIdx.x; k < n; k += stride) {
         const bool second = k >= n0;
         const InterpCell* cells = second ? A.fills[1].cells : A.fills[0].cells;

@@ -35,6 +35,7 @@
 //       3, split 27) less the 9 accumulations into zero; the update Q - l N   2 x 75 + 6 = 156
 //   PD  transverse differences, 3 x 8                                        24
 //   total 324 (the tile's halo adds about a third in the kernel).
+#include "claw_reflux.cuh"
 #include "claw_step.cuh"
 
 namespace claw {
@@ -103,14 +104,17 @@ __device__ __forceinline__ void tsplit(double d1, double d2, double d3, double u
 // STAGE: 0 cooperative loads, 1 tensor bulk copies (double buffered).  PULL: ghosts taken from
 // their source cells (separate instantiations, as for acoustics).
 template <int LIM, int TX, int TY, int NT, int STAGE, bool PULL>
-__global__ void __launch_bounds__(NT, 1) swe_step_kernel(const StepArgs A)
+__global__ void __launch_bounds__(NT, 1) swe_step_kernel(const __grid_constant__ StepArgs A)
 {
     using G = Geo<TX, TY>;
     using S = SweGeo<TX, TY>;
     constexpr int NBUF = STAGE ? 2 : 1;
     constexpr int NPER = (TX * TY + NT - 1) / NT;
-    if (A.step_grid && blockIdx.x >= A.step_grid) {   // a fill CTA (as in the acoustics kernel)
-        fill_jobs<NT>(A);
+    if (A.step_grid && blockIdx.x >= A.step_grid) {   // a CTA beside those (as in the acoustics kernel)
+        if (PULL == 0 && A.nreflux && blockIdx.x >= A.reflux_grid)   // (reflux levels fill their ghosts)
+            refl::run_jobs<LIM, NT>(A, A.reflux_grid, gridDim.x - A.reflux_grid);
+        else
+            fill_jobs<NT>(A);
         if (threadIdx.x == 0) finish_cta(A);
         return;
     }

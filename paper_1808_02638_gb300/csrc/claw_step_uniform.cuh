@@ -14,6 +14,7 @@
 #pragma once
 
 #include "claw_fixed.cuh"
+#include "claw_reflux.cuh"
 #include "claw_step.cuh"
 
 namespace claw {
@@ -237,8 +238,11 @@ __global__ void __launch_bounds__(NT, NT == 128 ? 4 : NT == 256 ? (TY == 16 ? 3 
     constexpr bool TWO = STAGE != 2;
     constexpr int NBUF = TWO ? 2 : 1;
     constexpr int NI = U::NI;
-    if (A.step_grid && blockIdx.x >= A.step_grid) {   // a fill CTA: no tiles, no shared memory
-        fill_jobs<NT>(A);
+    if (A.step_grid && blockIdx.x >= A.step_grid) {   // a CTA beside those: no tiles, no shared memory
+        if (PULL == 0 && A.nreflux && blockIdx.x >= A.reflux_grid)   // (reflux levels fill their ghosts)
+            refl::run_jobs<LIM, NT>(A, A.reflux_grid, gridDim.x - A.reflux_grid);
+        else
+            fill_jobs<NT>(A);
         if (threadIdx.x == 0) finish_cta(A);
         return;
     }

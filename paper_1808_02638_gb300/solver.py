@@ -341,11 +341,16 @@ class Hierarchy:
             if e is not None:
                 e.record()
             e = self._section("advance", stream)
-            if self.reflux and L > 0:             # this substep's fine fluxes at level L's interface
-                claw.claw_reflux_fine(self.ctx, L, q, cold, self.dt, self.rbuf[L], stream)
-            if self.reflux and L + 1 < self.nlev:  # the coarse fluxes at the finer level's interface
-                claw.claw_reflux_coarse(self.ctx, L + 1, q, self.dt, self.rbuf[L + 1], stream)
-            self.step_level(L, stream)
+            fine = self.rbuf[L] if self.reflux and L > 0 else None   # this substep's fine fluxes
+            coarse = self.rbuf[L + 1] if self.reflux and L + 1 < self.nlev else None   # the next interface's coarse ones
+            if self.reflux and not self.patchwise:   # in the step's own launch
+                claw.claw_level_step_reflux(self.ctx, L, q, dst, self.dt, self.smax, cold, fine, coarse, stream)
+            else:
+                if fine is not None:
+                    claw.claw_reflux_fine(self.ctx, L, q, cold, self.dt, fine, stream)
+                if coarse is not None:
+                    claw.claw_reflux_coarse(self.ctx, L + 1, q, self.dt, coarse, stream)
+                self.step_level(L, stream)
             if e is not None:
                 e.record()
         old, new = self.q[L][self.cur[L]], self.q[L][1 - self.cur[L]]
@@ -356,9 +361,11 @@ class Hierarchy:
                 filled = self.advance(L + 1, old, new, k / r, stream, filled=filled,
                                       tau_next=(k + 1) / r if k + 1 < r else None)
             e = self._section("update", stream)
-            claw.claw_average_down(self.ctx, L + 1, self.q[L + 1][self.cur[L + 1]], new, stream)
+            qf = self.q[L + 1][self.cur[L + 1]]
             if self.reflux:
-                claw.claw_reflux_apply(self.ctx, L + 1, self.rbuf[L + 1], self.dt, new, stream)
+                claw.claw_average_down_reflux(self.ctx, L + 1, qf, new, self.rbuf[L + 1], self.dt, stream)
+            else:
+                claw.claw_average_down(self.ctx, L + 1, qf, new, stream)
             if e is not None:
                 e.record()
         self.cur[L] ^= 1
