@@ -35,6 +35,9 @@
 //       3, split 27) less the 9 accumulations into zero; the update Q - l N   2 x 75 + 6 = 156
 //   PD  transverse differences, 3 x 8                                        24
 //   total 324 (the tile's halo adds about a third in the kernel).
+// The kernel issues fewer: reciprocals in three instructions (swe::recip), halvings and doublings in
+// the exponent field, h_p in three a wave, and a subcritical edge's side in 30 (PC).  2048^2 in patches of
+// 32^2: 3401 us a step before, 2900 now; it is bound by the FP64 pipe.
 #include "claw_reflux.cuh"
 #include "claw_step.cuh"
 
@@ -71,6 +74,44 @@ __device__ __forceinline__ double neg(double s) { return __double_as_longlong(s)
 __device__ __forceinline__ unsigned long long mag(double s)
 {
     return (unsigned long long)(__double_as_longlong(s) & 0x7fffffffffffffffLL);
+}
+
+// 1 / x for a positive normal x: the hardware's approximation (relative error below 2^-22) and one third-order
+// Newton (Householder) step, r (1 + e + e^2) with e = 1 - x r.  Three FP64 instructions, the last the
+// only rounding that shows (e^3 < 2^-66); the division routine takes five.
+__device__ __forceinline__ double recip(double x)
+{
+    double r;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+    const double e = fma(-x, r, 1.0);
+    return fma(r, fma(e, e, e), r);
+}
+// x / 2, 2 x for a normal x, in the exponent field (integer pipe)
+__device__ __forceinline__ double half(double x) { return __hiloint2double(__double2hiint(x) - 0x100000, __double2loint(x)); }
+__device__ __forceinline__ double twice(double x)   // (0 stays 0)
+{
+    const int hi = __double2hiint(x);
+    return __hiloint2double(hi + (hi & 0x7ff00000 ? 0x100000 : 0), __double2loint(x));
+}
+
+// tsplit for |un| < c, |ut| < c: the first transverse family goes down, the third up
+__device__ __forceinline__ void tsplit_sub(double d1, double d2, double d3, double un, double ut, double c,
+                                           double i2c, double* bm, double* bp)
+{
+    const double dh = d1 + d3;
+    const double t = d2 * i2c;
+    const double m1 = ut - c, m3 = ut + c;
+    const double g1 = m1 * fma(0.5, dh, -t), g3 = m3 * fma(0.5, dh, t), g2 = ut * (c * (d3 - d1));
+    const bool down = __double_as_longlong(ut) < 0;
+    bm[0] += g1;
+    bp[0] += g3;
+    bm[1] = fma(un, g1, bm[1]);
+    bp[1] = fma(un, g3, bp[1]);
+    const double a = (down ? bm[1] : bp[1]) + g2;
+    bm[1] = down ? a : bm[1];
+    bp[1] = down ? bp[1] : a;
+    bm[2] = fma(m1, g1, bm[2]);
+    bp[2] = fma(m3, g3, bp[2]);
 }
 
 // fluctuation with coefficients d1..d3 on the normal eigenvectors of an edge with Roe state
@@ -281,12 +322,12 @@ __global__ void __launch_bounds__(NT, 1) swe_step_kernel(const __grid_constant__
             for (int k = tid; k < n; k += NT) {
                 const int r = k / w + rx0, a = k - (r - rx0) * w - 1;
                 const int iR = (a + 2) + (r + 2) * G::SW, iL = iR - 1;
-                const double inv = 1.0 / (der[iL] + der[iR]);
+                const double inv = swe::recip(der[iL] + der[iR]);
                 const double un = (der[G::QPL + iL] + der[G::QPL + iR]) * inv;
                 const double ut = (der[2 * G::QPL + iL] + der[2 * G::QPL + iR]) * inv;
                 const double x = (sh[iL] + sh[iR]) * hg;
                 const double rc = rsqrt(x);
-                const double c = x * rc, i2c = 0.5 * rc;
+                const double c = x * rc, i2c = swe::half(rc);
                 const double dh = sh[iR] - sh[iL], dn = su[iR] - su[iL], dtg = sv[iR] - sv[iL];
                 const int e = (r + 1) * G::XEW + (a + 1);
                 XE[e] = un;
@@ -307,12 +348,12 @@ __global__ void __launch_bounds__(NT, 1) swe_step_kernel(const __grid_constant__
             for (int k = tid; k < n; k += NT) {
                 const int bb = k / w + by0, cc = k - (bb - by0) * w - 1;
                 const int iR = (cc + 2) + (bb + 2) * G::SW, iL = iR - G::SW;
-                const double inv = 1.0 / (der[iL] + der[iR]);
+                const double inv = swe::recip(der[iL] + der[iR]);
                 const double un = (der[2 * G::QPL + iL] + der[2 * G::QPL + iR]) * inv;
                 const double ut = (der[G::QPL + iL] + der[G::QPL + iR]) * inv;
                 const double x = (sh[iL] + sh[iR]) * hg;
                 const double rc = rsqrt(x);
-                const double c = x * rc, i2c = 0.5 * rc;
+                const double c = x * rc, i2c = swe::half(rc);
                 const double dh = sh[iR] - sh[iL], dn = sv[iR] - sv[iL], dtg = su[iR] - su[iL];
                 const int e = (bb + 1) * G::YEW + (cc + 1);
                 YE[e] = un;
@@ -346,7 +387,7 @@ __global__ void __launch_bounds__(NT, 1) swe_step_kernel(const __grid_constant__
             // 1 / (r1 . r1) and 1 / (r3 . r3) from one reciprocal of their product
             const double w = fma(ut, ut, 1.0);
             const double rr1 = fma(s1, s1, w), rr3 = fma(s3, s3, w);
-            const double ip = 1.0 / (rr1 * rr3);
+            const double ip = swe::recip(rr1 * rr3);
             double mu1, mu2, mu3;
             {   // wave 1 on (1, un - c, ut)
                 const double unI = E[u1], utI = E[plane + u1], cI = E[2 * plane + u1];
@@ -361,9 +402,9 @@ __global__ void __launch_bounds__(NT, 1) swe_step_kernel(const __grid_constant__
             }
             const double k1 = fabs(s1), k2 = fabs(un), k3 = fabs(s3);
             const double hl = -0.5 * l;
-            out[o] = fma(hl * k1, k1, 0.5 * k1) * mu1;
-            out[ol + o] = fma(hl * k2, k2, 0.5 * k2) * mu2;
-            out[2 * ol + o] = fma(hl * k3, k3, 0.5 * k3) * mu3;
+            out[o] = fma(hl, k1, 0.5) * (k1 * mu1);
+            out[ol + o] = fma(hl, k2, 0.5) * (k2 * mu2);
+            out[2 * ol + o] = fma(hl, k3, 0.5) * (k3 * mu3);
         };
         if (second) {
             if (carry)   // the carried limited x-edge rows, now that PA has read der
@@ -410,6 +451,38 @@ __global__ void __launch_bounds__(NT, 1) swe_step_kernel(const __grid_constant__
                     h2 = -h2;
                     h3 = -h3;
                 }
+            }
+            // subcritical along and across (decided by the edge alone, so that tilings and walks agree): the
+            // first wave goes left and down, the third right and up, and products with zero drop out: 30
+            // FP64 instructions a side instead of 42
+            if (swe::mag(un) < swe::mag(c) && swe::mag(ut) < swe::mag(c)) {
+                // the coefficients entering: e1 = h1, e3 = s3 a3 + h3 on the right (h with its sign), on the left
+                // e1 = s1 a1 + h1, e3 = h3; their transverse input adds hw h again
+                const double e2 = fma(right ? swe::pos(un) : swe::neg(un), a2, h2);
+                const double x = right ? fma(s3, a3, h3) : fma(s1, a1, h1);   // the wave that enters
+                const double y = right ? h1 : h3;                            // the other one's correction
+                if (nrm) {
+                    const double eh = x + y;
+                    nrm[0] += eh;
+                    nrm[1] = fma(right ? s3 : s1, x, fma(right ? s1 : s3, y, nrm[1]));
+                    nrm[2] = fma(ut, eh, nrm[2] + e2);
+                }
+                if (trans) {
+                    double dx = x, d2 = e2, dy = y;
+                    if (second) {
+                        if (hw > 0.0) {
+                            dx = x + (right ? h3 : h1);
+                            d2 = e2 + h2;
+                            dy = swe::twice(y);
+                        } else {
+                            dx = x - (right ? h3 : h1);
+                            d2 = e2 - h2;
+                            dy = 0.0;
+                        }
+                    }
+                    swe::tsplit_sub(right ? dy : dx, d2, right ? dx : dy, un, ut, c, i2c, bm, bp);
+                }
+                return;
             }
             const double e1 = fma(right ? swe::pos(s1) : swe::neg(s1), a1, h1);
             const double e2 = fma(right ? swe::pos(un) : swe::neg(un), a2, h2);
