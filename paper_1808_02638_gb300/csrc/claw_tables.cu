@@ -127,27 +127,97 @@ static void column_walks(const LevelDev& d, int piece, std::vector<TileDev>& out
     }
 }
 
-// tiles of a level for its tiling: sorted by area (largest first) for the persistent CTAs, or
-// as column walks (d.walk), and grouped by box for the per-box launches
+// Rows of the tiles a side of n cells is cut into, at most `most` each: full ones and a rest, or (even)
+// nearly equal ones.
+static int tile_rows(int n, int most, bool even)
+{
+    const int k = (n + most - 1) / most;
+    return even ? (n + k - 1) / k : most;
+}
+
+static void box_tiles(const claw_box& b, int n, int tx, int rows, std::vector<TileDev>& out)
+{
+    for (int y = 0; y < b.ny; y += rows)
+        for (int x = 0; x < b.nx; x += tx) {
+            TileDev T;
+            T.patch = n;
+            T.x0 = (short)x;
+            T.y0 = (short)y;
+            T.tx = (short)std::min(tx, b.nx - x);
+            T.ty = (short)std::min(rows, b.ny - y);
+            T.flags = 0;
+            out.push_back(T);
+        }
+}
+
+// Deals the tiles, largest first, to the SMs there and back (CTA i runs on SM i mod nsm, and steps tiles
+// i, i + grid, ...; grid is a multiple of nsm where it is below the number of tiles), so that an SM
+// with a large tile of one round has a small one of the next: an SM's FP64 pipe is shared by its
+// CTAs.  The last round, which may be short, goes forward.  (Shallow water on 169 boxes of 8 to 64
+// cells a side: an AMR coarse step of 42 level-steps took 3166 us with the tiles merely sorted, 3005
+// so.)
+static void deal(std::vector<TileDev>& t, int nsm)
+{
+    std::stable_sort(t.begin(), t.end(),
+                     [](const TileDev& a, const TileDev& b) { return (int)a.tx * a.ty > (int)b.tx * b.ty; });
+    for (size_t e = t.size() / nsm * nsm; e > 0; e -= std::min<size_t>(e, 2 * (size_t)nsm))
+        std::reverse(t.begin() + (e - nsm), t.begin() + e);
+}
+
+// The largest number of rows of a level's tiles, at most ty, for the kernels bound by the FP64 pipe: a
+// level of few tiles leaves SMs idle, or gives some two tiles and others one, and lower tiles fill
+// them.  The work of a tile is about its cells with the halo of its edges and a share for its
+// latency; the busiest SM decides.  Measured, full rows and lower ones: cell-wise medium 256^2
+// on 32 x 16 tiles 21.4 and 19.3 us (14 rows: 152 tiles for 152 SMs), 190 x 170 21.1 and 14.8 (8 rows); shallow
+// water 64^2 on 16 x 16 tiles 34.1 and 19 us (6 rows), 24 boxes with 14256 cells 35 and 24.  Past two
+// tiles an SM nothing is gained.  The uniform medium's integer step gains at most 3 % (100^2:
+// 6.4 and 6.2 us) and pays for halves of strips elsewhere: full rows there.
+static int choose_rows(const LevelDev& d, int tx, int ty, int nsm)
+{
+    long long full = 0;
+    for (const claw_box& b : d.boxes) full += (long long)((b.nx + tx - 1) / tx) * ((b.ny + ty - 1) / ty);
+    if (full > 2LL * nsm) return ty;   // (nothing gained: the rounds are many, the halo grows)
+    int best = ty;
+    double best_cost = 0.0;
+    std::vector<double> cost, sm(nsm);
+    for (int rows = ty; rows >= 4; rows -= std::max(1, rows / 8)) {
+        cost.clear();
+        for (const claw_box& b : d.boxes) {
+            const int h = tile_rows(b.ny, rows, rows < ty);
+            for (int y = 0; y < b.ny; y += h)
+                for (int x = 0; x < b.nx; x += tx)
+                    cost.push_back((std::min(tx, b.nx - x) + 2) * (std::min(h, b.ny - y) + 2.7) + 36.0);
+        }
+        if ((long long)cost.size() > 4LL * nsm) break;
+        std::sort(cost.begin(), cost.end(), [](double a, double b) { return a > b; });
+        std::fill(sm.begin(), sm.end(), 0.0);
+        const size_t rounds = (cost.size() + nsm - 1) / nsm;
+        for (size_t i = 0; i < cost.size(); ++i) {
+            const size_t k = i / nsm, r = i % nsm;
+            sm[(rounds - 1 - k) % 2 ? nsm - 1 - r : r] += cost[i];
+        }
+        const double c = *std::max_element(sm.begin(), sm.end());
+        if (rows == ty || c < 0.97 * best_cost) {
+            best = rows;
+            best_cost = c;
+        }
+    }
+    return best;
+}
+
+// tiles of a level for its tiling: dealt to the SMs by size for the persistent CTAs, or as column
+// walks (d.walk; full rows there), and grouped by box for the per-box launches
 int build_tiles(claw_ctx* ctx, int L)
 {
     LevelDev& d = ctx->lev[L];
     std::vector<TileDev> t;
     std::vector<int> start;
+    const bool fp64 = ctx->kind() != KIND_UNIFORM;
+    const int rows = fp64 ? choose_rows(d, d.tx, d.ty, std::max(1, ctx->nsm)) : d.ty;
     for (int n = 0; n < d.nboxes; ++n) {
         const claw_box& b = d.boxes[n];
         start.push_back((int)t.size());
-        for (int y = 0; y < b.ny; y += d.ty)
-            for (int x = 0; x < b.nx; x += d.tx) {
-                TileDev T;
-                T.patch = n;
-                T.x0 = (short)x;
-                T.y0 = (short)y;
-                T.tx = (short)std::min(d.tx, b.nx - x);
-                T.ty = (short)std::min(d.ty, b.ny - y);
-                T.flags = 0;
-                t.push_back(T);
-            }
+        box_tiles(b, n, d.tx, tile_rows(b.ny, rows, rows < d.ty), t);
     }
     start.push_back((int)t.size());
     // (the pieces are read by pack.commit: t keeps the box order, d.htiles the sorted copy)
@@ -167,9 +237,7 @@ int build_tiles(claw_ctx* ctx, int L)
         column_walks(d, piece, d.htiles, d.htcum);
     } else {
         d.htiles = t;
-        std::stable_sort(d.htiles.begin(), d.htiles.end(), [](const TileDev& a, const TileDev& b) {
-            return (int)a.tx * a.ty > (int)b.tx * b.ty;
-        });
+        deal(d.htiles, std::max(1, ctx->nsm));
     }
     d.ntiles = (int)d.htiles.size();
     for (auto& tm : ctx->tmaps[L]) cudaFree(tm.dev);
@@ -179,24 +247,12 @@ int build_tiles(claw_ctx* ctx, int L)
     if (d.walking) pack.add(&d.tcum, d.htcum);
     // adjoint tiles
     std::vector<TileDev> at;
-    const int e = adjoint_tile();
+    const int e = adjoint_tile(), arows = choose_rows(d, e, e, std::max(1, ctx->nsm));
     for (int n = 0; n < d.nboxes; ++n) {
         const claw_box& b = d.boxes[n];
-        for (int y = 0; y < b.ny; y += e)
-            for (int x = 0; x < b.nx; x += e) {
-                TileDev T;
-                T.patch = n;
-                T.x0 = (short)x;
-                T.y0 = (short)y;
-                T.tx = (short)std::min(e, b.nx - x);
-                T.ty = (short)std::min(e, b.ny - y);
-                T.flags = 0;
-                at.push_back(T);
-            }
+        box_tiles(b, n, e, tile_rows(b.ny, arows, arows < e), at);
     }
-    // largest first, like the step's tiles: the persistent CTAs end on small tiles
-    std::stable_sort(at.begin(), at.end(),
-                     [](const TileDev& a, const TileDev& b) { return (int)a.tx * a.ty > (int)b.tx * b.ty; });
+    deal(at, std::max(1, ctx->nsm));
     ctx->natiles[L] = (int)at.size();
     pack.add(&ctx->atiles[L], at);
     return pack.commit(d.tiletab);
