@@ -73,6 +73,7 @@ def time_tiling(H, L, tiling, reps=5, pull=False):
     for _ in range(2):
         claw.claw_level_advance(H.ctx, L, src, dst, H.aux[L], H.dt, smax, flags)
     e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+    torch.cuda._sleep(400_000)   # launches wait behind it: a level of 7 us is enqueued in more than it runs
     e0.record()
     for _ in range(reps):
         claw.claw_level_advance(H.ctx, L, src, dst, H.aux[L], H.dt, smax, flags)
