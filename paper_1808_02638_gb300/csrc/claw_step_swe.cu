@@ -36,8 +36,11 @@
 //   PD  transverse differences, 3 x 8                                        24
 //   total 324 (the tile's halo adds about a third in the kernel).
 // The kernel issues fewer: reciprocals in three instructions (swe::recip), halvings and doublings in
-// the exponent field, h_p in three a wave, and a subcritical edge's side in 30 (PC).  2048^2 in patches of
-// 32^2: 3401 us a step before, 2900 now; it is bound by the FP64 pipe.
+// the exponent field, a1 + a3 = dh, h_p in three a wave, and a subcritical edge's side in 30 (PC), four
+// less where the cell's sums start.  About 312 a cell with the halo of a 16 x 16 tile; 2048^2 in patches
+// of 32^2: 3401 us a step before, 2764 now, 90 % of the rate the FP64 pipe sustains.
+#include <type_traits>
+
 #include "claw_reflux.cuh"
 #include "claw_step.cuh"
 
@@ -88,13 +91,20 @@ __device__ __forceinline__ double recip(double x)
 }
 // x / 2, 2 x for a normal x, in the exponent field (integer pipe)
 __device__ __forceinline__ double half(double x) { return __hiloint2double(__double2hiint(x) - 0x100000, __double2loint(x)); }
+__device__ __forceinline__ double halve(double x)   // (0 stays 0)
+{
+    const int hi = __double2hiint(x);
+    return __hiloint2double(hi - (hi & 0x7fe00000 ? 0x100000 : 0), __double2loint(x));
+}
 __device__ __forceinline__ double twice(double x)   // (0 stays 0)
 {
     const int hi = __double2hiint(x);
     return __hiloint2double(hi + (hi & 0x7ff00000 ? 0x100000 : 0), __double2loint(x));
 }
 
-// tsplit for |un| < c, |ut| < c: the first transverse family goes down, the third up
+// tsplit for |un| < c, |ut| < c: the first transverse family goes down, the third up.  FIRST: bm and bp
+// are still zero and are set
+template <bool FIRST>
 __device__ __forceinline__ void tsplit_sub(double d1, double d2, double d3, double un, double ut, double c,
                                            double i2c, double* bm, double* bp)
 {
@@ -103,15 +113,15 @@ __device__ __forceinline__ void tsplit_sub(double d1, double d2, double d3, doub
     const double m1 = ut - c, m3 = ut + c;
     const double g1 = m1 * fma(0.5, dh, -t), g3 = m3 * fma(0.5, dh, t), g2 = ut * (c * (d3 - d1));
     const bool down = __double_as_longlong(ut) < 0;
-    bm[0] += g1;
-    bp[0] += g3;
-    bm[1] = fma(un, g1, bm[1]);
-    bp[1] = fma(un, g3, bp[1]);
+    bm[0] = FIRST ? g1 : bm[0] + g1;
+    bp[0] = FIRST ? g3 : bp[0] + g3;
+    bm[1] = FIRST ? un * g1 : fma(un, g1, bm[1]);
+    bp[1] = FIRST ? un * g3 : fma(un, g3, bp[1]);
     const double a = (down ? bm[1] : bp[1]) + g2;
     bm[1] = down ? a : bm[1];
     bp[1] = down ? bp[1] : a;
-    bm[2] = fma(m1, g1, bm[2]);
-    bp[2] = fma(m3, g3, bp[2]);
+    bm[2] = FIRST ? m1 * g1 : fma(m1, g1, bm[2]);
+    bp[2] = FIRST ? m3 * g3 : fma(m3, g3, bp[2]);
 }
 
 // fluctuation with coefficients d1..d3 on the normal eigenvectors of an edge with Roe state
@@ -334,12 +344,13 @@ __global__ void __launch_bounds__(NT, 1) swe_step_kernel(const __grid_constant__
                 XE[S::XE + e] = ut;
                 XE[2 * S::XE + e] = c;
                 XE[3 * S::XE + e] = i2c;
-                XE[4 * S::XE + e] = fma(un + c, dh, -dn) * i2c;
+                // a1 = ((un + c) dh - dn) / 2c, and a1 + a3 = dh
+                const double a1 = fma(fma(un, dh, -dn), i2c, swe::halve(dh));
+                XE[4 * S::XE + e] = a1;
                 XE[5 * S::XE + e] = fma(-ut, dh, dtg);
-                XE[6 * S::XE + e] = fma(-(un - c), dh, dn) * i2c;
+                XE[6 * S::XE + e] = dh - a1;
                 if (a >= 0 && a <= tx) {
-                    const unsigned long long s1 = swe::mag(un - c), s3 = swe::mag(un + c);
-                    m = umax64(m, umax64(s1, s3));
+                    m = umax64(m, swe::mag(fabs(un) + c));   // max(|un - c|, |un + c|), c > 0
                 }
             }
         }
@@ -360,12 +371,13 @@ __global__ void __launch_bounds__(NT, 1) swe_step_kernel(const __grid_constant__
                 YE[S::YE + e] = ut;
                 YE[2 * S::YE + e] = c;
                 YE[3 * S::YE + e] = i2c;
-                YE[4 * S::YE + e] = fma(un + c, dh, -dn) * i2c;
+                // a1 = ((un + c) dh - dn) / 2c, and a1 + a3 = dh
+                const double a1 = fma(fma(un, dh, -dn), i2c, swe::halve(dh));
+                YE[4 * S::YE + e] = a1;
                 YE[5 * S::YE + e] = fma(-ut, dh, dtg);
-                YE[6 * S::YE + e] = fma(-(un - c), dh, dn) * i2c;
+                YE[6 * S::YE + e] = dh - a1;
                 if (bb >= 0 && bb <= ty) {
-                    const unsigned long long s1 = swe::mag(un - c), s3 = swe::mag(un + c);
-                    m = umax64(m, umax64(s1, s3));
+                    m = umax64(m, swe::mag(fabs(un) + c));   // max(|un - c|, |un + c|), c > 0
                 }
             }
         }
@@ -436,8 +448,10 @@ __global__ void __launch_bounds__(NT, 1) swe_step_kernel(const __grid_constant__
         // is right of / above the edge).  Adds the normal-update part (A+dQ - F~ for the cell
         // on the right, A-dQ + F~ on the left; (h, n, t) components) to nrm and the transverse
         // split of the transverse input to bm / bp.
-        auto side = [&](const double* E, int plane, int e, const double* H, int lo, int lplane, bool right,
+        // The right one comes first: its sums start from zero.
+        auto side = [&](const double* E, int plane, int e, const double* H, int lo, int lplane, auto is_right,
                         double* nrm, double* bm, double* bp) {
+            constexpr bool right = decltype(is_right)::value;
             const double un = E[e], ut = E[plane + e], c = E[2 * plane + e], i2c = E[3 * plane + e];
             const double s1 = un - c, s3 = un + c;
             const double a1 = E[4 * plane + e], a2 = E[5 * plane + e], a3 = E[6 * plane + e];
@@ -462,10 +476,10 @@ __global__ void __launch_bounds__(NT, 1) swe_step_kernel(const __grid_constant__
                 const double x = right ? fma(s3, a3, h3) : fma(s1, a1, h1);   // the wave that enters
                 const double y = right ? h1 : h3;                            // the other one's correction
                 if (nrm) {
-                    const double eh = x + y;
-                    nrm[0] += eh;
-                    nrm[1] = fma(right ? s3 : s1, x, fma(right ? s1 : s3, y, nrm[1]));
-                    nrm[2] = fma(ut, eh, nrm[2] + e2);
+                    const double eh = x + y, sy = (right ? s1 : s3);
+                    nrm[0] = right ? eh : nrm[0] + eh;
+                    nrm[1] = fma(right ? s3 : s1, x, right ? sy * y : fma(sy, y, nrm[1]));
+                    nrm[2] = fma(ut, eh, right ? e2 : nrm[2] + e2);
                 }
                 if (trans) {
                     double dx = x, d2 = e2, dy = y;
@@ -480,7 +494,7 @@ __global__ void __launch_bounds__(NT, 1) swe_step_kernel(const __grid_constant__
                             dy = 0.0;
                         }
                     }
-                    swe::tsplit_sub(right ? dy : dx, d2, right ? dx : dy, un, ut, c, i2c, bm, bp);
+                    swe::tsplit_sub<right>(right ? dy : dx, d2, right ? dx : dy, un, ut, c, i2c, bm, bp);
                 }
                 return;
             }
@@ -507,8 +521,8 @@ __global__ void __launch_bounds__(NT, 1) swe_step_kernel(const __grid_constant__
         auto xcell = [&](int c, int r, double* nrm) {
             double bm[3] = {0.0, 0.0, 0.0}, bp[3] = {0.0, 0.0, 0.0};
             const int e = (r + 1) * G::XEW + (c + 1), lo = (r + 1) * G::XLW + c;
-            side(XE, S::XE, e, XH, lo, S::XL, true, nrm, bm, bp);
-            side(XE, S::XE, e + 1, XH, lo + 1, S::XL, false, nrm, bm, bp);
+            side(XE, S::XE, e, XH, lo, S::XL, std::true_type(), nrm, bm, bp);
+            side(XE, S::XE, e + 1, XH, lo + 1, S::XL, std::false_type(), nrm, bm, bp);
             if (trans) {   // (h, hu, hv) = (h, n, t)
                 const int d = (r + 1) * G::DW + c;
 #pragma unroll
@@ -522,8 +536,8 @@ __global__ void __launch_bounds__(NT, 1) swe_step_kernel(const __grid_constant__
         auto ycell = [&](int c, int r, double* nrm) {
             double bm[3] = {0.0, 0.0, 0.0}, bp[3] = {0.0, 0.0, 0.0};
             const int e = (r + 1) * G::YEW + (c + 1), lo = r * G::YLW + (c + 1);
-            side(YE, S::YE, e, YH, lo, S::YL, true, nrm, bm, bp);
-            side(YE, S::YE, e + G::YEW, YH, lo + G::YLW, S::YL, false, nrm, bm, bp);
+            side(YE, S::YE, e, YH, lo, S::YL, std::true_type(), nrm, bm, bp);
+            side(YE, S::YE, e + G::YEW, YH, lo + G::YLW, S::YL, std::false_type(), nrm, bm, bp);
             if (trans) {
                 const int d = r * G::EW + (c + 1);
                 Em[d] = bm[0];
