@@ -324,7 +324,7 @@ int claw_set_tiling(claw_ctx* ctx, int32_t L, int32_t tx, int32_t ty, int32_t st
                   (tx == 32 && ty == 32 && (threads == 0 || threads == 256 || threads == 512)) ||
                   (tx == 32 && ty == 16 && (threads == 0 || threads == 256)) ||
                   (tx == 16 && ty == 16 && (threads == 0 || threads == 128));
-    // staging 2 (one bulk-copy buffer, three CTAs per SM) exists for the acoustics 32x16 tiles
+    // staging 2 (one bulk-copy buffer) exists for the acoustics 32x16 tiles and the uniform medium's 32x32
     const bool staging2_ok = (ctx->kind() != KIND_SWE && tx == 32 && ty == 16 && (threads == 0 || threads == 256)) ||
                              (ctx->kind() == KIND_UNIFORM && tx == 32 && ty == 32 && (threads == 0 || threads == 256));
     if (!shape_ok || staging < 0 || staging > 2 || (staging == 2 && !staging2_ok) ||

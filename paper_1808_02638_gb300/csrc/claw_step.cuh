@@ -13,10 +13,11 @@
 //    loads;
 //  * every edge is solved once per tile; waves and fluctuations never leave shared memory;
 //    only Q^{n+1} is written back;
+//  * this file holds the cell-wise medium's kernel and what all step kernels share; the uniform
+//    medium's is claw_step_uniform.cuh, shallow water's claw_step_swe.cu;
 //  * the path is bound by the FP64 pipe (1/64 of FP32 on this part), so the arithmetic is
 //    arranged to minimise FP64 instructions: the transverse split is applied once per cell
-//    to the summed x-fluctuation (it is linear), constant coefficients fold into per-tile
-//    constants, limiters are division free (phi(b/a) a), wave speeds are reduced on the
+//    to the summed x-fluctuation (it is linear), limiters are division free (phi(b/a) a), wave speeds are reduced on the
 //    integer pipe as bit patterns;
 //  * the CFL reduction (Sec. 2.4, 3.2.2) is a warp-shuffle / shared-memory max per tile folded
 //    by the CTA, with one 64-bit atomic max per CTA and run on the run's device scalar.
