@@ -1,5 +1,5 @@
 // Dispatch of the fused level-step kernels (instantiated in claw_step_uniform.cu,
-// claw_step_cellwise.cu and claw_step_swe.cu).
+// claw_step_cellwise.cu and claw_step_swe.cuh).
 #include <algorithm>
 #include <mutex>
 #include <set>
@@ -9,7 +9,7 @@
 namespace claw {
 
 static StepKernel pick(int kind, int limiter, int tx, int ty, int nt, int staging, bool pull, bool rec = false,
-                       bool interp = false)
+                       bool interp = false, bool walk = false)
 {
     if (interp) {   // acoustics only; shallow water takes the interpolation launch first (claw_api.cu)
         if (!pull || rec) return StepKernel{nullptr, 0, 0};
@@ -30,6 +30,9 @@ static StepKernel pick(int kind, int limiter, int tx, int ty, int nt, int stagin
         return pull ? step_kernel_cellwise_pull(limiter, tx, ty, nt, staging)
                     : step_kernel_cellwise(limiter, tx, ty, nt, staging);
     case KIND_SWE:
+        if (walk)
+            return pull ? step_kernel_swe_pull_walk(limiter, tx, ty, nt, staging)
+                        : step_kernel_swe_walk(limiter, tx, ty, nt, staging);
         return pull ? step_kernel_swe_pull(limiter, tx, ty, nt, staging) : step_kernel_swe(limiter, tx, ty, nt, staging);
     }
     return StepKernel{nullptr, 0, 0};
@@ -47,7 +50,7 @@ static cudaError_t prepare(const StepKernel& k)
     auto key = std::make_pair((const void*)k.fn, dev);
     if (done.count(key)) return cudaSuccess;
     e = cudaFuncSetAttribute((const void*)k.fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)std::max(k.smem, k.smem_walk));
+                             (int)k.smem);
     if (e == cudaSuccess) done.insert(key);
     return e;
 }
@@ -55,10 +58,10 @@ static cudaError_t prepare(const StepKernel& k)
 int step_max_ctas_per_sm(int kind, int limiter, int tx, int ty, int nt, int staging, bool pull, bool rec, bool interp,
                          bool walk)
 {
-    StepKernel k = pick(kind, limiter, tx, ty, nt, staging, pull, rec, interp);
+    StepKernel k = pick(kind, limiter, tx, ty, nt, staging, pull, rec, interp, walk);
     if (!k.fn || prepare(k) != cudaSuccess) return 0;
     int n = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, (const void*)k.fn, k.nt, walk ? k.smem_walk : k.smem) !=
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, (const void*)k.fn, k.nt, k.smem) !=
         cudaSuccess)
         return 0;
     return n;
@@ -67,7 +70,8 @@ int step_max_ctas_per_sm(int kind, int limiter, int tx, int ty, int nt, int stag
 cudaError_t launch_step(const StepArgs& a, int kind, int limiter, int tx, int ty, int nt, int staging,
                         int grid, cudaStream_t s, int spare)
 {
-    StepKernel k = pick(kind, limiter, tx, ty, nt, staging, a.ring != nullptr, a.tape != nullptr, a.interp != nullptr);
+    StepKernel k = pick(kind, limiter, tx, ty, nt, staging, a.ring != nullptr, a.tape != nullptr, a.interp != nullptr,
+                        a.tcum != nullptr);
     if (!k.fn) return cudaErrorInvalidValue;
     cudaError_t e = prepare(k);
     if (e != cudaSuccess) return e;
@@ -82,13 +86,13 @@ cudaError_t launch_step(const StepArgs& a, int kind, int limiter, int tx, int ty
         b.step_grid = grid;
         const int extra = (int)std::min<long long>((items + k.nt - 1) / k.nt, std::max(spare, 1));
         b.reflux_grid = grid + extra;
-        k.fn<<<grid + extra + reflux, k.nt, a.tcum ? k.smem_walk : k.smem, s>>>(b);
+        k.fn<<<grid + extra + reflux, k.nt, k.smem, s>>>(b);
     } else if (reflux > 0) {
         StepArgs b = a;
         b.step_grid = b.reflux_grid = grid;
-        k.fn<<<grid + reflux, k.nt, a.tcum ? k.smem_walk : k.smem, s>>>(b);
+        k.fn<<<grid + reflux, k.nt, k.smem, s>>>(b);
     } else {
-        k.fn<<<grid, k.nt, a.tcum ? k.smem_walk : k.smem, s>>>(a);
+        k.fn<<<grid, k.nt, k.smem, s>>>(a);
     }
     return cudaGetLastError();
 }

@@ -813,7 +813,6 @@ struct StepKernel {
     void (*fn)(const StepArgs);
     size_t smem;        // dynamic shared memory of a launch
     int nt;
-    size_t smem_walk;   // ... of a launch that walks tile columns (shallow water: carried rows added)
 };
 
 template <int LIM, int TX, int TY, int NT, int STAGE, int PULL, bool REC = false>
@@ -821,7 +820,7 @@ StepKernel step_kernel_entry()
 {
     StepKernel k;
     k.fn = step_kernel<LIM, TX, TY, NT, STAGE, PULL, REC>;
-    k.smem = k.smem_walk = Geo<TX, TY>::smem_bytes(STAGE == 1 ? 2 : 1);
+    k.smem = Geo<TX, TY>::smem_bytes(STAGE == 1 ? 2 : 1);
     k.nt = NT;
     return k;
 }
@@ -844,7 +843,7 @@ StepKernel step_kernel_select(int tx, int ty, int nt, int staging)
     if (tx == 16 && ty == 16 && (nt == 0 || nt == 128))
         return staging ? step_kernel_entry<LIM, 16, 16, 128, 1, PULL, REC>()
                        : step_kernel_entry<LIM, 16, 16, 128, 0, PULL, REC>();
-    return StepKernel{nullptr, 0, 0, 0};
+    return StepKernel{nullptr, 0, 0};
 }
 
 template <int PULL, bool REC = false>
@@ -857,7 +856,7 @@ StepKernel step_kernel_for(int lim, int tx, int ty, int nt, int staging)
     case CLAW_LIM_VANLEER: return step_kernel_select<CLAW_LIM_VANLEER, PULL, REC>(tx, ty, nt, staging);
     case CLAW_LIM_MC: return step_kernel_select<CLAW_LIM_MC, PULL, REC>(tx, ty, nt, staging);
     }
-    return StepKernel{nullptr, 0, 0, 0};
+    return StepKernel{nullptr, 0, 0};
 }
 
 // one translation unit per kernel family (pull: the instantiations taking pulled ghosts)
@@ -871,5 +870,7 @@ StepKernel step_kernel_cellwise_record(int lim, int tx, int ty, int nt, int stag
 StepKernel step_kernel_cellwise_record_fill(int lim, int tx, int ty, int nt, int staging);
 StepKernel step_kernel_swe(int lim, int tx, int ty, int nt, int staging);
 StepKernel step_kernel_swe_pull(int lim, int tx, int ty, int nt, int staging);
+StepKernel step_kernel_swe_walk(int lim, int tx, int ty, int nt, int staging);
+StepKernel step_kernel_swe_pull_walk(int lim, int tx, int ty, int nt, int staging);
 
 }  // namespace claw

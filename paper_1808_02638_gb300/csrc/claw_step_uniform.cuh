@@ -497,7 +497,7 @@ template <int LIM, int TX, int TY, int NT, int STAGE, int PULL> StepKernel unifo
 {
     StepKernel k;
     k.fn = uniform_step_kernel<LIM, TX, TY, NT, STAGE, PULL>;
-    k.smem = k.smem_walk = UniGeo<TX, TY, NT>::smem(STAGE, PULL);
+    k.smem = UniGeo<TX, TY, NT>::smem(STAGE, PULL);
     k.nt = NT;
     return k;
 }
@@ -527,7 +527,7 @@ template <int LIM, int PULL> StepKernel uniform_kernel_select(int tx, int ty, in
     if (tx == 16 && ty == 16 && (nt == 0 || nt == 128))
         return staging ? uniform_kernel_entry<LIM, 16, 16, 128, 1, PULL>()
                        : uniform_kernel_entry<LIM, 16, 16, 128, 0, PULL>();
-    return StepKernel{nullptr, 0, 0, 0};
+    return StepKernel{nullptr, 0, 0};
 }
 
 template <int PULL> StepKernel uniform_kernel_for(int lim, int tx, int ty, int nt, int staging)
@@ -539,7 +539,7 @@ template <int PULL> StepKernel uniform_kernel_for(int lim, int tx, int ty, int n
     case CLAW_LIM_VANLEER: return uniform_kernel_select<CLAW_LIM_VANLEER, PULL>(tx, ty, nt, staging);
     case CLAW_LIM_MC: return uniform_kernel_select<CLAW_LIM_MC, PULL>(tx, ty, nt, staging);
     }
-    return StepKernel{nullptr, 0, 0, 0};
+    return StepKernel{nullptr, 0, 0};
 }
 
 }  // namespace claw

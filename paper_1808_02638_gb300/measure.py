@@ -27,7 +27,7 @@ from .solver import Hierarchy
 
 FP64_INSTR_UNIFORM = 42
 FP64_INSTR_CELLWISE = 78
-FP64_INSTR_SWE = 324     # shallow water, Roe solvers (claw_step_swe.cu states the count)
+FP64_INSTR_SWE = 324     # shallow water, Roe solvers (claw_step_swe.cuh states the count)
 BYTES_UNIFORM = 48.0
 BYTES_CELLWISE = 64.0
 FP64_ISSUE_PEAK_G = 152 * 2 * 2.07   # G FP64 instructions / s: 152 SMs x 2 per clock x 2.07 GHz
