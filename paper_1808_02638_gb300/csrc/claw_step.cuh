@@ -14,7 +14,7 @@
 //  * every edge is solved once per tile; waves and fluctuations never leave shared memory;
 //    only Q^{n+1} is written back;
 //  * this file holds the cell-wise medium's kernel and what all step kernels share; the uniform
-//    medium's is claw_step_uniform.cuh, shallow water's claw_step_swe.cu;
+//    medium's is claw_step_uniform.cuh, shallow water's claw_step_swe.cuh;
 //  * the path is bound by the FP64 pipe (1/64 of FP32 on this part), so the arithmetic is
 //    arranged to minimise FP64 instructions: the transverse split is applied once per cell
 //    to the summed x-fluctuation (it is linear), limiters are division free (phi(b/a) a), wave speeds are reduced on the

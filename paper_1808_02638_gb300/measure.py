@@ -10,7 +10,8 @@ ghost cells and halo recomputation are not counted), algorithmic HBM bytes per s
 and written, 48 B per cell-update; 64 B with the cell-wise medium's rho, K), the fraction of the
 measured copy bandwidth, and the fraction of the FP64 pipe's issue rate used by the algorithmic
 FP64 instructions of the step (42 per cell-update uniform, 78 cell-wise, 324 shallow water; the
-kernel sources state how they are counted).  Times are CUDA events around graph replays of whole coarse steps
+kernel sources state how they are counted; the uniform-medium step does most of its 42 in 64-bit
+integers, so its fraction may exceed 1).  Times are CUDA events around graph replays of whole coarse steps
 (ghost fill, every level-step with its substeps, averaging, the Eq. cfl update).
 """
 from __future__ import annotations
