@@ -407,9 +407,10 @@ __device__ __forceinline__ void pull_ghosts(const StepArgs& A, const PatchDev& P
 // The CTAs stride over the tiles by the grid (column walks are built for no cell-wise medium: its
 // ghost coefficients are the caller's and need not match the neighbour's interior).
 // Registers: the one-buffer staging is capped for three CTAs per SM; the 128-thread tiles for
-// five (the shared memory of five fits an SM), except those evaluating interpolated ghosts.
+// six (the shared memory of six fits an SM with one buffer; 16 two-level runs 3074 us a pass at five, 2905
+// at six).
 template <int LIM, int TX, int TY, int NT, int STAGE, int PULL, bool REC = false>
-__global__ void __launch_bounds__(NT, STAGE == 2 ? 3 : (NT == 128 && !REC ? 5 : 1))
+__global__ void __launch_bounds__(NT, STAGE == 2 ? 3 : (NT == 128 && !REC ? 6 : 1))
     step_kernel(const StepArgs A)
 {
     using G = Geo<TX, TY>;
