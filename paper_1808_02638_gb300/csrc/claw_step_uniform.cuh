@@ -19,12 +19,6 @@
 
 namespace claw {
 
-__device__ __forceinline__ void cp_async8(void* dst, const void* src)
-{
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(smem_u32(dst)), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
-
 // rows that the FP64 phases step at a time (their work arrays then fit the fixed-point tile's)
 constexpr int kFp64Rows = 8;
 
