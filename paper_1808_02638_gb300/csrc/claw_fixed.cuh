@@ -10,8 +10,8 @@
 // fused multiply-add per component).
 //
 // Precision: with e the smallest exponent such that |du|, |dv|, |dp| / Z < 2^e on every edge of the
-// tile, the unit is 2^(e - 58).  Sums and limiters are exact, a product errs by less than 2.5
-// units, and the increment of a cell by a few units: about 2^-56 of the tile's largest jump, where
+// tile, the unit is 2^(e - 58).  Sums and limiters are exact, a product errs by at most
+// 0.75 units, and the increment of a cell by a few units: about 2^-56 of the tile's largest jump, where
 // a double's rounding is 2^-53 of the value at hand.  A tile is stepped this way only if at every
 // edge the state next to it or the jump across it is at least 2^(e - 4): the error then is below
 // the rounding of the local state.  Every other tile (a state on a zero background in front of a
@@ -24,7 +24,7 @@
 //
 // What bounds it: the integer pipes (about 1.8 instructions an SM and clock of 4, the ALU busiest), no longer
 // FP64 or memory.  2048^2 in patches of 32^2 with pulled ghosts, MC limiter: 412 us a step with the
-// FP64 phases, 185 now; 777 x 555 in ragged patches, van Leer: 146 and 44 (the FP64 reciprocals went).
+// FP64 phases, 193 now; 1001 x 604 in ragged patches, van Leer: 146 and 47 (the FP64 reciprocals went).
 #pragma once
 
 #include "claw_internal.h"
@@ -34,40 +34,60 @@ namespace fx {
 
 // ------------------------------------------------------------------------- numbers
 // a constant c in [0, 1/4]: c = (hi 2^32 + lo) / 2^64, lo signed, 0 <= hi <= 2^30
-struct Coef {
+struct __align__(16) Coef {
     int hi, lo;
+    unsigned half;   // 2^31 + lo / 2: half a unit, and the mean of the product that mul drops
 };
 __device__ __forceinline__ Coef coef_bits(long long c)   // c 2^64, at most 2^62
 {
     Coef r;
     r.lo = (int)(unsigned)c;
     r.hi = (int)((c - r.lo) >> 32);
+    r.half = 0x80000000u + (unsigned)(r.lo >> 1);
     return r;
 }
 
-// v c from 2.5 units below to half a unit above: of the two cross products only the upper words are
-// formed (each rounded down) and the product of the low words, below half a unit, is dropped.  0 gives
-// 0: where nothing changes, nothing may.
+// Rounding: products and conversions are of magnitudes, to nearest, and take the sign afterwards; quarters
+// round halves to even.  Results are then odd functions of their arguments, so that a mirror-symmetric
+// state stays so bit for bit, and their errors have no preferred sign.  Rounding downwards instead (184
+// against 193 us a step of 2048^2) let the total of p drift by 6e-15 a step on 64^2 cells, linearly; like
+// this it wanders no further than that of the FP64 phases.
+
+// w c for a magnitude w < 2^63, within 0.75 units: the product of the low words, between -1/2 and 1/2 units,
+// is replaced by its mean.  0 gives 0: where nothing changes, nothing may.
+__device__ __forceinline__ long long mul_mag(long long w, Coef c)
+{
+    const int wh = (int)(w >> 32);
+    long long x = (long long)wh * c.lo + (long long)(unsigned long long)c.half;   // cross products, units / 2^32
+    x += (long long)((unsigned long long)(unsigned)w * (unsigned)c.hi);           // below 2^62 each
+    return (long long)wh * c.hi + (int)(x >> 32);
+}
+// m with its sign changed if s < 0.  (A select: exclusive or and difference took 203 against 193 us a step of
+// 2048^2.)
+__device__ __forceinline__ long long signed_by(long long m, int s) { return s < 0 ? -m : m; }
+__device__ __forceinline__ int sign_of(long long v) { return (int)(v >> 32); }
+__device__ __forceinline__ int sign_of(double d) { return __double2hiint(d); }
 __device__ __forceinline__ long long mul(long long v, Coef c)
 {
-    const int vh = (int)(v >> 32);
-    const int t = __mulhi(vh, c.lo) + (int)__umulhi((unsigned)v, (unsigned)c.hi);   // |.| <= 2^30 each
-    return (long long)vh * c.hi + t;
+    const int s = sign_of(v);
+    return signed_by(mul_mag(signed_by(v, s), c), s);
 }
+// v / 4, halves to even
+__device__ __forceinline__ long long quarter(long long v) { return (v + 1 + ((v >> 2) & 1)) >> 2; }
 
 __device__ __forceinline__ unsigned mag_hi(double x) { return (unsigned)__double2hiint(x) & 0x7fffffffu; }
 
-// d 2^(L + 1075 - base) truncated towards zero, for a finite d whose biased exponent is at most
-// base (base >= 64: zeros and subnormals give 0)
-template <int L> __device__ __forceinline__ long long from_double(double d, int base)
+// |d| 2^(L + 1075 - base) for a finite d whose biased exponent is at most base (base >= 64: zeros and
+// subnormals give 0), to nearest (halves up) or truncated
+template <int L, bool NEAREST> __device__ __forceinline__ long long mag_from_double(double d, int base)
 {
     const int hi = __double2hiint(d);
     const int e = (hi >> 20) & 0x7ff;
     unsigned long long m =
         ((unsigned long long)(unsigned)((hi & 0xfffff) | 0x100000) << 32) | (unsigned)__double2loint(d);
-    m <<= L;
+    m <<= NEAREST ? L + 1 : L;
     asm("shr.u64 %0, %0, %1;" : "+l"(m) : "r"(base - e));   // clamps at 64: no test of the amount
-    return hi < 0 ? -(long long)m : (long long)m;
+    return (long long)(NEAREST ? (m + 1) >> 1 : m);
 }
 
 // the double nearest to v, |v| < 2^62 (halves away from zero)
@@ -83,40 +103,33 @@ __device__ __forceinline__ double to_double(long long v)
 }
 
 // ------------------------------------------------------------------------- limiters
-// lim2<L>(a, b) = 2 phi(b / a) a, exact.  With s the sign of a (0 or -1), x = a ^ s and y = b ^ s are
-// the magnitudes of values with a's sign, less one for negative ones; y < 0: the signs differ (or
-// b = 0 with a < 0).  Doubling such a magnitude shifts s in from below, and a sum of two adds -s.
-// van Leer's quotient is rounded (see below).
+// Lim2<L>::f(x, y) = 2 phi(y / x) x for x >= 0 and y of either sign, exact (van Leer's quotient is rounded,
+// see below): the limited strength of a = x with its neighbour upwind b = y, both with a's sign taken out.
 template <int L> struct Lim2;
 template <> struct Lim2<CLAW_LIM_NONE> {
-    static __device__ __forceinline__ long long f(long long a, long long) { return a + a; }
+    static __device__ __forceinline__ long long f(long long x, long long) { return x + x; }
 };
 template <> struct Lim2<CLAW_LIM_MINMOD> {
-    static __device__ __forceinline__ long long f(long long a, long long b)
+    static __device__ __forceinline__ long long f(long long x, long long y)
     {
-        const long long s = a >> 63, x = a ^ s, y = b ^ s;
-        const long long r = (((x < y ? x : y) << 1) | (s & 1)) ^ s;
+        const long long r = (x < y ? x : y) << 1;
         return y < 0 ? 0 : r;
     }
 };
 template <> struct Lim2<CLAW_LIM_SUPERBEE> {
-    static __device__ __forceinline__ long long f(long long a, long long b)
-    {   // max(min(|a|, 2 |b|), min(2 |a|, |b|))
-        const long long s = a >> 63, x = a ^ s, y = b ^ s;
-        const long long x2 = (x << 1) | (s & 1), y2 = (y << 1) | (s & 1);
+    static __device__ __forceinline__ long long f(long long x, long long y)
+    {   // 2 max(min(x, 2 y), min(2 x, y))
+        const long long x2 = x << 1, y2 = y << 1;
         const long long m1 = x < y2 ? x : y2, m2 = x2 < y ? x2 : y;
-        const long long m = m1 > m2 ? m1 : m2;
-        const long long r = ((m << 1) | (s & 1)) ^ s;
+        const long long r = (m1 > m2 ? m1 : m2) << 1;
         return y < 0 ? 0 : r;
     }
 };
 template <> struct Lim2<CLAW_LIM_MC> {
-    static __device__ __forceinline__ long long f(long long a, long long b)
-    {   // min(|a| + |b|, 4 min(|a|, |b|))
-        const long long s = a >> 63, x = a ^ s, y = b ^ s;
-        const long long t = x + y - s;
-        const long long q = ((x < y ? x : y) << 2) | (s & 3);
-        const long long r = (t < q ? t : q) ^ s;
+    static __device__ __forceinline__ long long f(long long x, long long y)
+    {   // min(x + y, 4 min(x, y))
+        const long long t = x + y, q = (x < y ? x : y) << 2;
+        const long long r = t < q ? t : q;
         return y < 0 ? 0 : r;
     }
 };
@@ -127,10 +140,8 @@ template <> struct Lim2<CLAW_LIM_MC> {
 // 2^-60, the result (at most 2^60) by at most seven units; an integer or FP64 division would cost
 // several times the 65 instructions.
 template <> struct Lim2<CLAW_LIM_VANLEER> {
-    static __device__ __forceinline__ long long f(long long a, long long b)
+    static __device__ __forceinline__ long long f(long long x, long long y)
     {
-        const long long s = a >> 63;
-        const long long x = (a ^ s) - s, y = (b ^ s) - s;
         const unsigned long long lo = (unsigned long long)(x < y ? x : y), hi = (unsigned long long)(x < y ? y : x);
         const int sh = __clzll((long long)(lo + hi)) - 3;   // x + y < 2^60 and not 0 where the result is used
         const unsigned long long sn = (lo + hi) << (sh & 63), ln = lo << (sh & 63);
@@ -149,15 +160,22 @@ template <> struct Lim2<CLAW_LIM_VANLEER> {
         const unsigned hh = (unsigned)(h >> 32), hl = (unsigned)h, fh = (unsigned)(f >> 32), fl = (unsigned)f;
         const unsigned c = __umulhi(hh, fl) + __umulhi(hl, fh);   // below 2^31 each
         const long long m = (long long)((unsigned long long)hh * fh + c);   // 4 max(x, y) f
-        return x > 0 && y > 0 ? (m ^ s) - s : 0;
+        return x > 0 && y > 0 ? m : 0;
     }
 };
+
+// c 2 phi(b / a) a
+template <int L> __device__ __forceinline__ long long limited(long long a, long long b, Coef c)
+{
+    const int s = sign_of(a);
+    return signed_by(mul_mag(Lim2<L>::f(signed_by(a, s), signed_by(b, s)), c), s);
+}
 
 // ------------------------------------------------------------------------- shared state of a CTA
 struct Shared {
     unsigned mp[2], mu[2];   // per tile parity: largest high words of |dp|, of |du| and |dv|
     int mn[2];               // smallest high word of the local magnitude of an edge (wave units)
-    int iz_exp;              // 1 / Z0 = f 2^iz_exp, f in [1, 2); iz = f / 8
+    int iz_exp;              // 1 / Z0 = f 2^iz_exp, f in [1, 2); iz = f / 32
     Coef iz;
     // constants of a run, written by thread 0; two sets, so that one can be written while the
     // CTA's other threads finish a tile with the other
@@ -178,7 +196,7 @@ __device__ __forceinline__ void init(Shared& S, double iZ)
     S.mn[0] = S.mn[1] = 0x7fffffff;
     const long long b = __double_as_longlong(iZ);
     S.iz_exp = (int)((b >> 52) & 0x7ff) - 1023;
-    S.iz = coef_bits(((b & 0xfffffffffffffLL) | (1LL << 52)) << 9);
+    S.iz = coef_bits(((b & 0xfffffffffffffLL) | (1LL << 52)) << 7);
 }
 
 // by a whole warp, a lane per constant (one thread forming all five held up a lone tile by 3800
@@ -249,18 +267,17 @@ template <int R> __device__ __forceinline__ long long last_row(const long long (
 //
 // Units and ranges, U = 2^58 the bound of |du|, |dv|, |dp| / Z and A = 2 U that of the strengths:
 //   a1, a2 = du -+ dp / Z                                          A = 2^59
-//   M = 2 phi a, S = M2 - M1, P = M1 + M2                          4 A
+//   M = (1 - nu) / 4 2 phi a, S = M2 - M1, P = M1 + M2             A
 //   ap = A2_w + A1_e, au = A2_w - A1_e                             2 A
-//   bp = S_e - S_w, bu = P_e - P_w   (twice the limited jumps)     8 A = 2^62
-//   m = (1 - nu) bp / 4, n = (1 - nu) bu / 4                       2 A
+//   m = S_e - S_w, n = P_e - P_w   (k, l of the y-edges)           2 A
 //   D / 4 = (ap + 2 m) / 4  (x-fluctuation pressure; E likewise)   3/2 A
 //   X = ap + m, U = au + n of the x-edges, Y, V of the y-edges    4 A
 // and with Q4 = (D_n + D_s - 2 D + E_e + E_w - 2 E) / 4 (below 12 A < 2^63) the increments are
 //   p / Z  -1/2 (nu_x X + nu_y Y + nu_x nu_y Q4)
 //   u      -nu_x / 2 (U - nu_y (E_e - E_w) / 4),   v  -nu_y / 2 (V - nu_x (D_n - D_s) / 4)
 // The larger nu of p and the nu in front of u and v are left to the fused multiply-add that adds the
-// increment to q (in FP64, with a quarter of the bracket as its integer operand), so that square
-// cells take no product for them and others one.
+// increment to q (in FP64, with the bracket, of p a quarter of it, as its integer operand: below 5 A
+// and 7 A), so that square cells take no product for them and others one.  4 (E_e - E_w) is below 12 A.
 template <class G, int LIM, int TX, int TY, int NT, bool KEEP, class Jumps, class Begin, class Strengths,
           class Limited>
 __device__ __forceinline__ bool step_tile(const StepArgs& A, const PatchDev& P, Shared& sh, const Shared::Run& run,
@@ -367,12 +384,14 @@ __device__ __forceinline__ bool step_tile(const StepArgs& A, const PatchDev& P, 
         const Coef iz = sh.iz;
 #pragma unroll
         for (int j = 0; j < R; ++j) {
-            const long long tx_ = mul(from_double<7>(xp[j], bp), iz), dx = from_double<5>(xu[j], e);
+            const long long tx_ = signed_by(mul_mag(mag_from_double<9, false>(xp[j], bp), iz), sign_of(xp[j]));
+            const long long dx = signed_by(mag_from_double<5, true>(xu[j], e), sign_of(xu[j]));
             a1[j] = dx - tx_;
             a2[j] = dx + tx_;
             A1[j * NT] = a1[j];
             A2[j * NT] = a2[j];
-            const long long ty_ = mul(from_double<7>(yp[j], bp), iz), dy = from_double<5>(yv[j], e);
+            const long long ty_ = signed_by(mul_mag(mag_from_double<9, false>(yp[j], bp), iz), sign_of(yp[j]));
+            const long long dy = signed_by(mag_from_double<5, true>(yv[j], e), sign_of(yv[j]));
             b1[j] = dy - ty_;
             b2[j] = dy + ty_;
         }
@@ -395,12 +414,13 @@ __device__ __forceinline__ bool step_tile(const StepArgs& A, const PatchDev& P, 
             bp[j] = b2[j] + b1n;
             bv[j] = b2[j] - b1n;
             if (second) {
-                const long long m1 = Lim2<LIM>::f(a1[j], a1e);   // left-going: upwind edge to the right
-                const long long m2 = Lim2<LIM>::f(a2[j], A2[j * NT - 1]);
+                const Coef cx = run.c[C_DX], cy = run.c[C_DY];
+                const long long m1 = limited<LIM>(a1[j], a1e, cx);   // left-going: upwind edge to the right
+                const long long m2 = limited<LIM>(a2[j], A2[j * NT - 1], cx);
                 SX[j * NT] = m2 - m1;
                 PX[j * NT] = m1 + m2;
-                const long long n1 = Lim2<LIM>::f(b1[j], b1n);
-                const long long n2 = Lim2<LIM>::f(b2[j], below(b2, j, b2d));
+                const long long n1 = limited<LIM>(b1[j], b1n, cy);
+                const long long n2 = limited<LIM>(b2[j], below(b2, j, b2d), cy);
                 sy[j] = n2 - n1;
                 py[j] = n1 + n2;
                 if (j == 0) {
@@ -415,26 +435,26 @@ __device__ __forceinline__ bool step_tile(const StepArgs& A, const PatchDev& P, 
 
     // ---------------------------------------------------------------- per-cell terms
     // the exchange slots of a1, a2 are free: E goes to A1, D of a strip's first and last row to A2
-    long long hp[R], hu[R], hv[R], d4[R], e4[R];   // a quarter of the brackets; D / 4, E / 4
+    long long hp[R], hu[R], hv[R], d4[R], e4[R];   // the brackets (of p: a quarter); D / 4, E / 4
     {
         const long long syu = second && up ? SY[w] : 0, pyu = second && up ? PY[w] : 0;
 #pragma unroll
         for (int j = 0; j < R; ++j) {
             long long m = 0, n = 0, k = 0, l = 0;
             if (second) {
-                m = mul(SX[j * NT + 1] - SX[j * NT], run.c[C_DX]);
-                n = mul(PX[j * NT + 1] - PX[j * NT], run.c[C_DX]);
-                k = mul(above(sy, j, rows, syu) - sy[j], run.c[C_DY]);
-                l = mul(above(py, j, rows, pyu) - py[j], run.c[C_DY]);
+                m = SX[j * NT + 1] - SX[j * NT];
+                n = PX[j * NT + 1] - PX[j * NT];
+                k = above(sy, j, rows, syu) - sy[j];
+                l = above(py, j, rows, pyu) - py[j];
             }
             const long long X = ap[j] + m, Y = bp[j] + k;
-            if (run.steep == 0) hp[j] = (X + Y) >> 2;
-            else if (run.steep == 1) hp[j] = (X >> 2) + mul(Y, run.c[C_RATIO]);
-            else hp[j] = (Y >> 2) + mul(X, run.c[C_RATIO]);
-            hu[j] = (au[j] + n) >> 2;
-            hv[j] = (bv[j] + l) >> 2;
-            d4[j] = (ap[j] + (cw ? m + m : 0)) >> 2;
-            e4[j] = (bp[j] + (cw ? k + k : 0)) >> 2;
+            if (run.steep == 0) hp[j] = quarter(X + Y);
+            else if (run.steep == 1) hp[j] = quarter(X) + mul(Y, run.c[C_RATIO]);
+            else hp[j] = quarter(Y) + mul(X, run.c[C_RATIO]);
+            hu[j] = au[j] + n;
+            hv[j] = bv[j] + l;
+            d4[j] = quarter(ap[j] + (cw ? m + m : 0));
+            e4[j] = quarter(bp[j] + (cw ? k + k : 0));
             if (trans) {
                 A1[j * NT] = e4[j];
             }
@@ -449,8 +469,8 @@ __device__ __forceinline__ bool step_tile(const StepArgs& A, const PatchDev& P, 
     // ---------------------------------------------------------------- update, store
     if (nr > 0 && a >= 0 && a < tx) {
         const double unit2 = -__hiloint2double((e - 56) << 20, 0);   // -2^(e - 1079), twice the unit
-        const double ku = run.nux * unit2, kv = run.nuy * unit2;
-        const double kp = Z0 * (run.steep == 2 ? kv : ku);
+        const double kx = run.nux * unit2, ky = run.nuy * unit2;
+        const double kp = Z0 * (run.steep == 2 ? ky : kx), ku = 0.25 * kx, kv = 0.25 * ky;
         const int W = P.nx + 4;
         const long long WH = (long long)W * (P.ny + 4);
         double* dst = A.qnew + P.qoff + (long long)(y0 + r0 + 2) * W + (x0 + a + 2);
@@ -463,8 +483,8 @@ __device__ __forceinline__ bool step_tile(const StepArgs& A, const PatchDev& P, 
                 const long long ds = below(d4, j, dd);
                 const long long ee = A1[j * NT + 1], ew = A1[j * NT - 1];
                 hp[j] += mul((dn + ds) + (ee + ew) - 2 * (d4[j] + e4[j]), run.c[C_MIN]);
-                hu[j] -= mul(ee - ew, run.c[C_NY]);
-                hv[j] -= mul(dn - ds, run.c[C_NX]);
+                hu[j] -= mul((ee - ew) << 2, run.c[C_NY]);
+                hv[j] -= mul((dn - ds) << 2, run.c[C_NX]);
             }
             const double* s = sp + (a + 2) + (r0 + j + 2) * G::SW;
             const double p = fma(to_double(hp[j]), kp, KEEP ? q[KEEP ? j : 0][0] : s[0]);
