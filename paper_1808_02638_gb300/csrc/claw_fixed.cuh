@@ -9,18 +9,29 @@
 // where the result is formed: the jumps dp, du, dv (rounded as before) and q + increment (one
 // fused multiply-add per component).
 //
-// Precision: with e the smallest exponent such that |du|, |dv|, |dp| / Z < 2^e on every edge of the
-// tile, the unit is 2^(e - 58).  Sums and limiters are exact, a product errs by at most
-// 0.75 units, and the increment of a cell by a few units: about 2^-56 of the tile's largest jump, where
-// a double's rounding is 2^-53 of the value at hand.  A tile is stepped this way only if at every
-// edge the state next to it or the jump across it is at least 2^(e - 4): the error then is below
-// the rounding of the local state.  Every other tile (a state on a zero background in front of a
-// wave, infinities, NaN, extreme exponents, a CFL number above 1 in either direction) takes the
-// FP64 phases.  The choice depends on the tile's states alone, so the result does not depend on
-// how the tile was staged or who stepped it.  Why 2^(e - 4): the
-// increment errs by a few units, some 2^(e - 56), which is the rounding (2^-52) of a state that large;
-// measured against 64-bit references the fixed-point step errs by 1.1e-16 where the FP64 phases err by
-// 1.5e-16, and a tile sent to the FP64 phases takes 2.2 times as long.
+// Precision: with e such that |du|, |dv|, |dp| / Z < 2^e on every edge of the tile, by their exponents and that
+// of 1 / Z, the unit is 2^(e - 58).  Sums and limiters are exact (van Leer's quotient within 7 units of
+// M, see below), a product errs by at most 0.75 units.  An increment of p / Z, u or v errs by up to 5
+// units, 1.3 rms (emulated, uniformly random states with exact jumps: all limiters, orders and
+// transverse modes); the bound by adding all up is 25.
+//
+// A tile is stepped this way only if at every edge the state next to it or the jump across it, the largest
+// of |p| / Z, |u| and |v|, is at least 2^(e - 4): 5 units are then 2.5 roundings (2^-53) of that state, and
+// the fused multiply-add that forms the result is the one other.  The FP64 phases take five such
+// operations for p and three for u and v.  Emulated, relative to the state, in cells beside a
+// jump at that limit: at most 2.4 and 1.7 roundings (p; u and v), 0.72 and 0.58 rms, where the FP64 phases
+// have 4.4 and 2.9, 1.2 and 0.94.  The first-order step has two and one operations without transverse
+// terms (2.0 and 1.0 roundings at most; fixed point 1.5 and 1.2 at 2^(e - 4)): it takes fixed point
+// from 2^(e - 2) on.
+//
+// The precision is that of the state as a vector in wave units.  A component far smaller than the others and
+// than the tile's jumps (a transverse velocity of 1e-9 beside jumps of 0.1 in p) is stepped to the same
+// absolute error, 2^-56 of the largest jump, not to its own last bits as in FP64.
+//
+// Every other tile (a state on a zero background in front of a wave, infinities, NaN, extreme exponents, a CFL
+// number above 1 in either direction) takes the FP64 phases, 2.1 times as long.  Path and unit
+// depend on the states of the tile alone: how it was staged or who stepped it does not matter, but
+// its shape does.  Two tilings of the same state agree to rounding, not bit for bit.
 //
 // What bounds it: the integer pipes (about 1.8 instructions an SM and clock of 4, the ALU busiest), no longer
 // FP64 or memory.  2048^2 in patches of 32^2 with pulled ghosts, MC limiter: 412 us a step with the
@@ -373,7 +384,8 @@ __device__ __forceinline__ bool step_tile(const StepArgs& A, const PatchDev& P, 
     int e = max((int)(mu >> 20), mp ? (int)(mp >> 20) + sh.iz_exp + 1 : 0);
     bool fine = run.ok && mp < 0x7ff00000u && mu < 0x7ff00000u;
     if ((mp | mu) == 0u) e = 1023;   // no jump above 2^-1042: every fixed-point jump is 0
-    fine = fine && e >= 500 && e <= 1600 && (mn >> 20) >= ((mp | mu) ? e - 3 : 100);
+    const int least = second ? e - 3 : e - 1;   // biased exponent: 2^(e - 4) and 2^(e - 2) of the bound
+    fine = fine && e >= 500 && e <= 1600 && (mn >> 20) >= ((mp | mu) ? least : 100);
     if (!fine) return false;
     begin();
 
