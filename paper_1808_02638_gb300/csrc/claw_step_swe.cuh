@@ -85,15 +85,17 @@ __device__ __forceinline__ unsigned long long mag(double s)
     return (unsigned long long)(__double_as_longlong(s) & 0x7fffffffffffffffLL);
 }
 
-// 1 / x for a positive normal x: the hardware's approximation (relative error below 2^-22) and one third-order
-// Newton (Householder) step, r (1 + e + e^2) with e = 1 - x r.  Three FP64 instructions, the last the
-// only rounding that shows (e^3 < 2^-66); the division routine takes five.
+// 1 / x for x in [2^-1022, 2^1022]; +-0 for an infinity, NaN for NaN and 0.  rcp.approx.ftz.f64 sees the upper 20
+// mantissa bits of x and returns as many, so |e| = |1 - x r| < 2^-19, and one third-order Newton
+// (Householder) step, r (1 + e + e^2), leaves e^3 < 2^-57 beside the last operation's rounding.  Three FP64
+// instructions; the division routine, correctly rounded, takes five.
 __device__ __forceinline__ double recip(double x)
 {
     double r;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
     const double e = fma(-x, r, 1.0);
-    return fma(r, fma(e, e, e), r);
+    const double y = fma(r, fma(e, e, e), r);
+    return (__double2hiint(x) & 0x7fffffff) == 0x7ff00000 ? r : y;   // (an infinity: e is NaN; NaNs here are quiet)
 }
 // wave strengths of an edge from its Roe state (s1, s3 = un -+ c, ut, i2c = 1 / (2 c)) and jumps of (h, normal,
 // tangential momentum).  a3 is not formed as dh - a1, an instruction less: where the third wave is all but
@@ -106,12 +108,19 @@ __device__ __forceinline__ void strengths(double s1, double s3, double ut, doubl
     a2 = fma(-ut, dh, dt);
     a3 = fma(-s1, dh, dn) * i2c;
 }
-// x / 2, 2 x for a normal x, in the exponent field (integer pipe)
-__device__ __forceinline__ double half(double x) { return __hiloint2double(__double2hiint(x) - 0x100000, __double2loint(x)); }
-__device__ __forceinline__ double twice(double x)   // (0 stays 0)
+// x / 2 and 2 x in the exponent field (integer pipe), for 0 and where x and the result are normal; infinities and
+// NaN stay what they are
+__device__ __forceinline__ int exponent_step(double x)   // 0x100000, but 0 for 0, subnormals, infinities and NaN
 {
-    const int hi = __double2hiint(x);
-    return __hiloint2double(hi + (hi & 0x7ff00000 ? 0x100000 : 0), __double2loint(x));
+    return (unsigned)((__double2hiint(x) & 0x7fffffff) - 0x100000) < 0x7fe00000u ? 0x100000 : 0;
+}
+__device__ __forceinline__ double half(double x)
+{
+    return __hiloint2double(__double2hiint(x) - exponent_step(x), __double2loint(x));
+}
+__device__ __forceinline__ double twice(double x)
+{
+    return __hiloint2double(__double2hiint(x) + exponent_step(x), __double2loint(x));
 }
 
 // tsplit for |un| < c, |ut| < c: the first transverse family goes down, the third up.  FIRST: bm and bp
