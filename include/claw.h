@@ -322,7 +322,8 @@ int claw_unpack_interiors(claw_ctx* ctx, int32_t level, int32_t box_begin, int32
  * need_start[k + 1]) (those holding its boxes and the cells its ghosts come from) have arrived.  Copies
  * and steps run on streams of the context beside `stream`, which they start from and are joined to;
  * no buffer may be reused before `stream` has passed that point.  Calls on one context share those
- * streams.  Errors: CLAW_EINVAL, CLAW_ENOMEM, CLAW_ECUDA. */
+ * streams.  Errors: CLAW_EINVAL (also for a piece that ends behind the packed interiors), CLAW_ENOMEM,
+ * CLAW_ECUDA. */
 int claw_steps_from_host(claw_ctx* ctx, double* q0, double* q1, const double* aux, double* dt, double* smax,
                          double* host_a, double* host_b, double* stage_in, double* stage_out,
                          int32_t nsteps, int32_t npieces, const int32_t* piece_boxes,

@@ -51,9 +51,12 @@ extern "C" int claw_steps_from_host(claw_ctx* ctx, double* q0, double* q1, const
     if (!valid_level(ctx, 0) || !q0 || !q1 || !dt || !smax || !host_a || !host_b || nsteps < 0 || npieces < 1 ||
         !piece_boxes || !ranges || !need_start || !needs || (stage_in == nullptr) != (stage_out == nullptr))
         return CLAW_EINVAL;
+    // a packed buffer holds the level's packed interiors; how far a pool reaches only the caller knows
+    const int64_t most = stage_in ? (int64_t)ctx->lev[0].packed : INT64_MAX / (int64_t)sizeof(double);
     for (int k = 0; k < npieces; ++k) {
         if (piece_boxes[k] < 0 || piece_boxes[k + 1] < piece_boxes[k] || piece_boxes[k + 1] > ctx->lev[0].nboxes ||
-            ranges[2 * k] < 0 || ranges[2 * k + 1] < ranges[2 * k] || need_start[k + 1] < need_start[k])
+            ranges[2 * k] < 0 || ranges[2 * k + 1] < ranges[2 * k] || ranges[2 * k + 1] > most || need_start[k] < 0 ||
+            need_start[k + 1] < need_start[k])
             return CLAW_EINVAL;
         for (int m = need_start[k]; m < need_start[k + 1]; ++m)
             if (needs[m] < 0 || needs[m] >= npieces) return CLAW_EINVAL;
