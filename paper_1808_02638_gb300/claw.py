@@ -143,10 +143,8 @@ def _ptr(t):
     return t.data_ptr()
 
 
-def _host(t):
-    """host pointer of a contiguous double tensor"""
-    if t.is_cuda:
-        raise ValueError("a host tensor is wanted")
+def _mem(t):
+    """pointer of a torch tensor, in host memory or on a device"""
     return t.data_ptr()
 
 
@@ -394,14 +392,14 @@ def claw_unpack_interiors(ctx, level, box_begin, box_end, packed, q, stream=None
 def claw_steps_from_host(ctx, q0, q1, aux, dt, smax, host_a, host_b, stage_in, stage_out, nsteps, pieces, ranges,
                          needs, stream=None):
     """pieces: [(first box, end box)], contiguous; ranges: [(begin, end)] elements of a host buffer;
-    needs: [[pieces]]"""
+    needs: [[pieces]].  host_a, host_b: contiguous doubles, in host memory or on a device"""
     import numpy as np
     boxes = np.array([a for a, _ in pieces] + [pieces[-1][1]], dtype=np.int32)
     rng = np.array(ranges, dtype=np.int64).reshape(-1)
     start = np.cumsum([0] + [len(n) for n in needs]).astype(np.int32)
     flat = np.array([m for n in needs for m in n], dtype=np.int32)
     _check("claw_steps_from_host", load().claw_steps_from_host(
-        ctx, _ptr(q0), _ptr(q1), _ptr(aux), _ptr(dt), _ptr(smax), _host(host_a), _host(host_b), _ptr(stage_in),
+        ctx, _ptr(q0), _ptr(q1), _ptr(aux), _ptr(dt), _ptr(smax), _mem(host_a), _mem(host_b), _ptr(stage_in),
         _ptr(stage_out), int(nsteps), len(pieces), boxes.ctypes.data, rng.ctypes.data, start.ctypes.data,
         flat.ctypes.data, _stream(stream)))
 

@@ -418,18 +418,24 @@ class Hierarchy:
         pieces, one below 3 MB of host buffer.  Measured, us a step of a packed state of 1.6 MB (256^2):
         66 in one piece, 71 in four; 6.3 MB: 127, 114 and 157 in eight; 25 MB: 359, 221, 236; 101 MB
         (2048^2): 1316, 676, 704 (a piece costs the host 13 us, a step in one piece overlaps
-        nothing).  Returns the host buffer holding the final state."""
+        nothing).  The buffers may be longer than the state (host_b) and of any kind that Tensor.copy_
+        takes: pageable, on a device, or, through pinned doubles and with a synchronisation at the
+        end, of other types and strides.  Returns the host buffer holding the final state."""
         if self.nlev != 1 or self.nruns != 1:
             raise ValueError("host-resident stepping is for one-level hierarchies of one run")
-        plain = all(t.dtype == torch.float64 and t.is_contiguous() for t in (host_a, host_b))
-        if not plain:   # other types and strides go through plain buffers
-            a, b = (torch.empty(host_a.numel(), dtype=torch.float64).pin_memory() for _ in range(2))
-            a.copy_(host_a)
+        n = host_a.numel()
+        if host_b.numel() < n:
+            raise ValueError("host_b must be as long as host_a")
+        if not all(t.dtype == torch.float64 and t.is_contiguous() for t in (host_a, host_b)):
+            a, b = (torch.empty(n, dtype=torch.float64, pin_memory=True) for _ in range(2))
+            a.copy_(host_a.detach().reshape(-1))
             out = self.steps_from_host(a, b, nsteps, bands)
             torch.cuda.current_stream(self.dev).synchronize()
-            host_a.copy_(a)
-            if nsteps:
-                host_b.copy_(b)
+            # (what the steps did not write stays untouched: it need not be writable)
+            for t, v, first in ((host_b, b, 1), (host_a, a, 2)):
+                if nsteps >= first:
+                    part = t if t.numel() == n else t[:n]
+                    part.copy_(v.view(part.shape))
             return host_a if out is a else host_b
         packed = host_a.numel() == self.packed_size(0)
         if bands is None:
@@ -448,16 +454,19 @@ class Hierarchy:
             stage = self._stage
         elif host_a.numel() != self.q[0][0].numel():
             raise ValueError("host buffers must hold the level's pool or its packed interiors")
-        if host_b.numel() != host_a.numel():
-            raise ValueError("host buffers must have the same length")
+        if nsteps <= 0:
+            return host_a
         c = self.cur[0]
         with torch.cuda.device(self.dev):
-            claw.claw_steps_from_host(self.ctx, self.q[0][c], self.q[0][1 - c], self.aux[0], self.dt, self.smax,
-                                      host_a, host_b, *stage, nsteps, parts, ranges, needs)
-            # torch's allocators learn that the buffers are in use up to here on this stream
-            for t in (host_a, host_b):
-                if t.is_pinned():
-                    torch.empty(1, dtype=torch.float64, device=self.dev).copy_(t.view(-1)[:1], non_blocking=True)
+            try:
+                claw.claw_steps_from_host(self.ctx, self.q[0][c], self.q[0][1 - c], self.aux[0], self.dt, self.smax,
+                                          host_a, host_b, *stage, nsteps, parts, ranges, needs)
+            finally:
+                # torch's allocators learn that the buffers are in use up to here on this stream (also when
+                # the call failed after its first copies)
+                for t in (host_a, host_b):
+                    if not t.is_cuda and t.is_pinned():
+                        torch.empty(1, dtype=torch.float64, device=self.dev).copy_(t.view(-1)[:1], non_blocking=True)
         self.cur[0] ^= nsteps & 1
         return host_b if nsteps & 1 else host_a
 
