@@ -13,9 +13,11 @@ workload (same metric and unit).
 from __future__ import annotations
 
 import argparse
+import hashlib
 import json
 import math
 import os
+import re
 import statistics
 import subprocess
 import sys
@@ -51,9 +53,7 @@ BYTES_PER_CELL = 48.0     # read q^n (p, u, v) + write q^{n+1}: algorithmic HBM 
 # clock: 152 SMs x 2 x 2.07 GHz = 629 G instructions/s; 1.259 TFLOP/s if all were FMAs.
 FP64_ISSUE_PEAK_G = 152 * 2 * 2.07
 FP64_PEAK_TFLOPS = 152 * 2 * 2 * 2.07e9 / 1e12
-# The pipe the kernel is bound by: integer ALU instructions executed per cell (profiler counters of the
-# 32 x 32 tile, halo included) against 64 lanes per SM per clock (LOP3 measures 65).
-ALU_INSTR_PER_CELL = 444
+# The integer ALU pipe that the kernel uses most: 64 lanes per SM per clock (LOP3 measures 65).
 ALU_PEAK_G = 152 * 64 * 2.07
 
 
@@ -63,6 +63,42 @@ def measured_peaks():
             return json.load(f)
     except OSError:
         return {}
+
+
+# ----------------------------------------------------------------- profiler record
+def kernel_sources(root=ROOT):
+    """the benchmark kernel's translation unit and every header that it includes, sorted"""
+    csrc = os.path.join(root, "paper_1808_02638_gb300", "csrc")
+    todo, seen = ["claw_step_uniform_pull.cu"], set()
+    while todo:
+        name = todo.pop()
+        if name in seen:
+            continue
+        seen.add(name)
+        with open(os.path.join(csrc, name)) as f:
+            todo += re.findall(r'^#include "(claw_[^"/]+)"', f.read(), re.M)
+    return [os.path.join(csrc, n) for n in sorted(seen)]
+
+
+def kernel_hash(root=ROOT):
+    h = hashlib.sha256()
+    for path in kernel_sources(root):
+        with open(path, "rb") as f:
+            h.update(os.path.basename(path).encode() + b"\0" + f.read() + b"\0")
+    return h.hexdigest()[:16]
+
+
+def profiled_launch(tiling, root=ROOT):
+    """the profiler's record of the benchmark's launch (DRAM bytes, executed instructions), or None if it
+    was taken of another tiling or of other sources"""
+    try:
+        with open(os.path.join(root, "profiles", "step_uniform_2048x2048_traffic.json")) as f:
+            rec = json.load(f)
+        if rec.get("source_sha256_16") == kernel_hash(root) and rec.get("tiling") == list(tiling):
+            return rec
+    except (OSError, ValueError):
+        pass
+    return None
 
 
 # ----------------------------------------------------------------- clocks
@@ -438,23 +474,17 @@ def main():
     peaks = measured_peaks()
     hbm = peaks.get("hbm_gbs", 6800.0)
     achieved_gops = ALG_FP64_INSTR_PER_CELL * N_CELLS / kern_avg_s / 1e9
-    alu_gops = ALU_INSTR_PER_CELL * N_CELLS / kern_avg_s / 1e9
     achieved_tflops = ALG_FLOPS_PER_CELL * N_CELLS / kern_avg_s / 1e12
     achieved_gbs = BYTES_PER_CELL * N_CELLS / kern_avg_s / 1e9
-    # DRAM traffic of one launch from the last profiler capture, only while the kernel source
-    # is unchanged since that capture
-    traffic = None
-    tf = os.path.join(ROOT, "profiles", "step_uniform_2048x2048_traffic.json")
-    if os.path.exists(tf):
-        try:
-            import hashlib
-            rec = json.load(open(tf))
-            src = b"".join(open(os.path.join(ROOT, "paper_1808_02638_gb300", "csrc", f), "rb").read()
-                           for f in ("claw_fixed.cuh", "claw_step_uniform.cuh"))
-            if hashlib.sha256(src).hexdigest()[:16] == rec.get("source_sha256_16"):
-                traffic = rec.get("bytes_per_launch")
-        except (OSError, ValueError):
-            traffic = None
+    # what a profiler counted on one launch of this kernel, if this is the kernel
+    rec = profiled_launch(tiling)
+    executed = None
+    if rec:
+        alu_gops = rec["alu_instructions_per_cell"] * N_CELLS / kern_avg_s / 1e9
+        executed = {"alu_instructions_per_cell": rec["alu_instructions_per_cell"], "alu_ginstr": alu_gops,
+                    "alu_pipe_ginstr": ALU_PEAK_G, "frac": alu_gops / ALU_PEAK_G,
+                    "note": "integer ALU instructions executed, halo included (profiler); the pipe: 152 SMs x 64 "
+                            "lanes/clk x 2.07 GHz (derived; independent LOP3 loops measured 65 per SM per clk)"}
     line = {
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": K,
         "warmup": args.warmup, "ms_per_step": total_ms / K, "higher_is_better": True, "scaling": "weak",
@@ -467,17 +497,16 @@ def main():
         "step": "one CUDA-graph replay of the persistent level-step launch (all 4096 patches, each tile's "
                 "ghosts pulled from their source cells, Eq. cfl on the last CTA)",
         "ghosts": "pulled by the step kernel from their source cells (no ghost-copy launch)",
-        "roofline": {"bound": "alu", "achieved": alu_gops, "peak": ALU_PEAK_G,
-                     "unit": "G integer ALU instructions/s", "frac": alu_gops / ALU_PEAK_G, "traffic": traffic,
-                     "per_cell_update": f"{ALU_INSTR_PER_CELL} integer ALU instructions executed; the method: "
-                                        f"{ALG_FP64_INSTR_PER_CELL} FP64 instructions (25 DADD + 17 DFMA), "
+        "roofline": {"bound": "latency of integer chains", "achieved": achieved_gbs, "peak": hbm,
+                     "unit": "GB/s (algorithmic bytes)", "frac": achieved_gbs / hbm,
+                     "traffic": rec["bytes_per_launch"] if rec else None,
+                     "per_cell_update": f"the method: {ALG_FP64_INSTR_PER_CELL} FP64 instructions (25 DADD + 17 DFMA), "
                                         f"{ALG_FLOPS_PER_CELL} flops, {BYTES_PER_CELL:.0f} B",
                      "kernel": "level-step (uniform medium, MC), autotuned tiling "
                                f"{tiling[0]}x{tiling[1]} tiles, {tiling[3]} threads, "
                                f"{STAGINGS[tiling[2]]} staging",
                      "kernel_ms": kern_avg_s * 1e3,
-                     "peak_source": "ALU pipe: 152 SMs x 64 lanes/clk x 2.07 GHz (derived; independent LOP3 loops "
-                                    "measured 65 per SM per clk)",
+                     "executed": executed,
                      "method_fp64": {"achieved_ginstr": achieved_gops, "fp64_pipe_ginstr": FP64_ISSUE_PEAK_G,
                                      "note": "above the FP64 pipe's rate: the step works in 64-bit integers"},
                      "flops": {"achieved_tflops": achieved_tflops, "peak_tflops": FP64_PEAK_TFLOPS,
