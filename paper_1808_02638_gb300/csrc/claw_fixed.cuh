@@ -28,14 +28,15 @@
 // than the tile's jumps (a transverse velocity of 1e-9 beside jumps of 0.1 in p) is stepped to the same
 // absolute error, 2^-56 of the largest jump, not to its own last bits as in FP64.
 //
-// Every other tile (a state on a zero background in front of a wave, infinities, NaN, extreme exponents, a CFL
-// number above 1 in either direction) takes the FP64 phases, 2.1 times as long.  Path and unit
-// depend on the states of the tile alone: how it was staged or who stepped it does not matter, but
-// its shape does.  Two tilings of the same state agree to rounding, not bit for bit.
+// Every other tile (a front on a zero background, infinities, NaN, extreme exponents, a CFL number above 1 in
+// either direction) takes the FP64 phases, 2.5 times as long; a tile without any jump does not, whatever its
+// state.  Path and unit depend on the states of the tile alone: how it was staged or who stepped it does
+// not matter, but its shape does.  Two tilings of the same state agree to rounding, not bit for bit.
 //
-// What bounds it: the integer pipes (about 1.8 instructions an SM and clock of 4, the ALU busiest), no longer
-// FP64 or memory.  2048^2 in patches of 32^2 with pulled ghosts, MC limiter: 412 us a step with the
-// FP64 phases, 193 now; 1001 x 604 in ragged patches, van Leer: 146 and 47 (the FP64 reciprocals went).
+// What bounds it: the latency of dependent integer chains at 16 warps an SM; no pipe is at its limit (the ALU
+// is the busiest), and FP64 and memory no longer are.  2048^2 in patches of 32^2 with pulled ghosts, MC
+// limiter: 412 us a step when all of it was FP64, 193 now; 1001 x 604 in ragged patches, van Leer: 146 and
+// 47 (the FP64 reciprocals went).
 #pragma once
 
 #include "claw_internal.h"
@@ -163,7 +164,8 @@ template <> struct Lim2<CLAW_LIM_VANLEER> {
         const unsigned long long e = (1ull << 63) - (unsigned long long)v0 * d;
         const unsigned v = v0 + (__umulhi((unsigned)(e >> 11), v0) >> 20);
         const unsigned q1 = __umulhi((unsigned)(ln >> 29), v);   // f 2^31
-        const unsigned long long p1 = (unsigned long long)q1 * (unsigned)sn + ((unsigned long long)(q1 * (unsigned)(sn >> 32)) << 32);
+        const unsigned long long p1 =
+            (unsigned long long)q1 * (unsigned)sn + ((unsigned long long)(q1 * (unsigned)(sn >> 32)) << 32);
         const long long rem = (long long)((ln << 31) - p1);      // (f 2^31 - q1) sn, |.| < 2^63
         const long long p2 = (long long)(int)(rem >> 32) * (int)(v >> 1);   // rem / sn 2^59
         const unsigned long long f = ((unsigned long long)q1 << 31) + (unsigned long long)(p2 >> 28);   // f 2^62
@@ -188,7 +190,7 @@ struct Shared {
     int mn[2];               // smallest high word of the local magnitude of an edge (wave units)
     int iz_exp;              // 1 / Z0 = f 2^iz_exp, f in [1, 2); iz = f / 32
     Coef iz;
-    // constants of a run, written by thread 0; two sets, so that one can be written while the
+    // constants of a run, written by the last warp; two sets, so that one can be written while the
     // CTA's other threads finish a tile with the other
     struct Run {
         Coef c[6];           // see C_DX ..; nu = dt c0 / h
@@ -210,7 +212,7 @@ __device__ __forceinline__ void init(Shared& S, double iZ)
     S.iz = coef_bits(((b & 0xfffffffffffffLL) | (1LL << 52)) << 7);
 }
 
-// by a whole warp, a lane per constant (one thread forming all five held up a lone tile by 3800
+// by a whole warp, a lane per constant (one thread forming all of them held up a lone tile by 3800
 // cycles, most of a third of it)
 __device__ __forceinline__ void init_run(const Shared& S, Shared::Run& R, double dt, double dxinv, double dyinv,
                                          double c0)
@@ -273,8 +275,8 @@ template <int R> __device__ __forceinline__ long long last_row(const long long (
 // staged tile is read before the first barrier only (the next tile's copy may land in it behind
 // that); otherwise it is read again at the end.  `jumps_done` is called before the
 // first barrier and, on the fixed-point path, `begin` behind it, `strengths_done` before the
-// second and `limited_done` before the third: the fetches for the next tile.  What the last phase reads of the exchange slots is next written behind two barriers of the
-// next tile, so no barrier ends the tile.
+// second and `limited_done` before the third: the fetches for the next tile.  What the last phase reads of
+// the exchange slots is next written behind two barriers of the next tile, so no barrier ends the tile.
 //
 // Units and ranges, U = 2^58 the bound of |du|, |dv|, |dp| / Z and A = 2 U that of the strengths:
 //   a1, a2 = du -+ dp / Z                                          A = 2^59
@@ -386,6 +388,18 @@ __device__ __forceinline__ bool step_tile(const StepArgs& A, const PatchDev& P, 
     if ((mp | mu) == 0u) e = 1023;   // no jump above 2^-1042: every fixed-point jump is 0
     const int least = second ? e - 3 : e - 1;   // biased exponent: 2^(e - 4) and 2^(e - 2) of the bound
     fine = fine && e >= 500 && e <= 1600 && (mn >> 20) >= ((mp | mu) ? least : 100);
+    if (!fine && run.ok && (mp | mu) == 0u) {
+        // a tile whose jumps are zero to the last bit comes out as it is, in integers as in FP64, however small its
+        // state.  (Zeros in front of a wave, the whole of 2048^2: 507 us by the FP64 phases, 217 so.)
+        bool still = true;
+#pragma unroll
+        for (int j = 0; j < R; ++j) {
+            const bool in = j < nr;
+            if (in && r0 + j <= ty) still = still && xp[j] == 0.0 && xu[j] == 0.0;
+            if (in && a <= tx) still = still && yp[j] == 0.0 && yv[j] == 0.0;
+        }
+        fine = !__syncthreads_or(!still);
+    }
     if (!fine) return false;
     begin();
 

@@ -19,36 +19,39 @@
 
 namespace claw {
 
-// rows that the FP64 phases step at a time (their work arrays then fit the fixed-point tile's)
-constexpr int kFp64Rows = 8;
-
-template <int TX, int TY, int NT> struct UniGeo {
+// Rows that the FP64 phases step at a time: 16 where that costs the kernel nothing, since the halo rows and the
+// barriers then weigh less (2048^2, MC, every tile sent there, us a step by 8 and 16 rows: 32 x 32 tiles
+// 516 and 474, 16 x 16 with 128 threads 544 and 491).  The others would lose a CTA per SM to the
+// larger work arrays (32 x 16, two buffers) or spill under their register caps (32 x 16 with 352
+// threads 236 and 299 in fixed point, 16 x 16 with 192 threads 255 and 273).
+template <int TX, int TY, int NT, int STAGE> struct UniGeo {
     using G = Geo<TX, TY>;
+    static constexpr int FP64_ROWS = TX == TY && NT != 192 ? 16 : 8;
     static constexpr int NF = 4 * (TX + TY + 4);             // cells of a staged tile's two-cell frame
     static constexpr int NI = (NF + NT - 1) / NT;            // ... of one thread
-    static constexpr int FP64 = Geo<TX, kFp64Rows>::NWORK, FIXED = fx::Strips<TX, TY, NT>::WORDS;
+    static constexpr int FP64 = Geo<TX, FP64_ROWS>::NWORK, FIXED = fx::Strips<TX, TY, NT>::WORDS;
     static constexpr int WORK = ((FP64 > FIXED ? FP64 : FIXED) + 15) / 16 * 16;
     // q buffers, work arrays, side buffer of the pulled frame, two barriers (8-byte words)
-    static constexpr int side(int stage, int pull) { return pull && stage == 2 ? 3 * NF : 0; }
-    static constexpr size_t smem(int stage, int pull)
+    static constexpr int side(int pull) { return pull && STAGE == 2 ? 3 * NF : 0; }
+    static constexpr size_t smem(int pull)
     {
-        return (size_t)((stage == 2 ? 1 : 2) * G::QSTRIDE + WORK + side(stage, pull) + 2) * 8;
+        return (size_t)((STAGE == 2 ? 1 : 2) * G::QSTRIDE + WORK + side(pull) + 2) * 8;
     }
 };
 
 // ------------------------------------------------------------------------- the FP64 phases
-// Steps the staged tile (planes qpl apart, rows SW = TX + 4) into q_new in rounds of kFp64Rows rows;
+// Steps the staged tile (planes qpl apart, rows SW = TX + 4) into q_new in rounds of ROWS rows;
 // returns the error flags seen.  With a = 2 alpha and M = phi(theta) a:
 //   x-normal update  dp = -(lx K/2) ap - (lx kap Z/4) bp,  du = -(lx c/2) au - (lx kap/4) bu
 //   (dp also carries the centre term 2 kT D of the transverse update)
 //   ap = A2_w + A1_e, au = A2_w - A1_e, bp = S_e - S_w, bu = P_e - P_w,  kap = c (1 - lx c)
 //   x-fluctuation pressure into the cell D = (K/2) (ap + (1 - lx c) bp)
-template <int LIM, int TX, int NT>
+template <int LIM, int TX, int ROWS, int NT>
 __device__ __noinline__ int uniform_tile_fp64(const StepArgs& A, const PatchDev& P, const double* sq, int qpl,
                                               double* work, int tx, int tile_ty, int x0, int tile_y0)
 {
-    using G = Geo<TX, kFp64Rows>;
-    constexpr int NPER = (TX * kFp64Rows + NT - 1) / NT;
+    using G = Geo<TX, ROWS>;
+    constexpr int NPER = (TX * ROWS + NT - 1) / NT;
     double* A1x = work;                             // x-edge wave strengths, family 1 / 2
     double* A2x = A1x + G::XEW * G::XEH;
     double* B1y = A2x + G::XEW * G::XEH;            // y-edge wave strengths
@@ -89,8 +92,8 @@ __device__ __noinline__ int uniform_tile_fp64(const StepArgs& A, const PatchDev&
         s_k[10] = -kT;
         s_k[11] = trans ? 0.125 * lx * ly * c0 * c0 : 0.0;   // kU
     }
-    for (int h0 = 0; h0 < tile_ty; h0 += kFp64Rows) {
-        const int ty = min(kFp64Rows, tile_ty - h0), y0 = tile_y0 + h0;
+    for (int h0 = 0; h0 < tile_ty; h0 += ROWS) {
+        const int ty = min(ROWS, tile_ty - h0), y0 = tile_y0 + h0;
         const double* sp = sq + h0 * G::SW;
         const double* su = sp + qpl;
         const double* sv = su + qpl;
@@ -152,7 +155,7 @@ __device__ __noinline__ int uniform_tile_fp64(const StepArgs& A, const PatchDev&
             dP[n] = dU[n] = dV[n] = 0.0;
             const int ci = tid + n * NT;
             const int c = ci % TX, r = ci / TX;
-            if (ci >= TX * kFp64Rows || c >= tx || r >= ty) continue;
+            if (ci >= TX * ROWS || c >= tx || r >= ty) continue;
             const int iq = (c + 2) + (r + 2) * G::SW;
             const int ex = (r + 1) * G::XEW + (c + 1);
             const int ey = (r + 1) * G::YEW + (c + 1);
@@ -198,7 +201,7 @@ __device__ __noinline__ int uniform_tile_fp64(const StepArgs& A, const PatchDev&
         for (int n = 0; n < NPER; ++n) {
             const int ci = tid + n * NT;
             const int c = ci % TX, r = ci / TX;
-            if (ci >= TX * kFp64Rows || c >= tx || r >= ty) continue;
+            if (ci >= TX * ROWS || c >= tx || r >= ty) continue;
             double p = dP[n], u = dU[n], v = dV[n];
             if (trans) {
                 const double dn = Dx[(r + 2) * G::DW + c], ds = Dx[r * G::DW + c];
@@ -219,15 +222,15 @@ __device__ __noinline__ int uniform_tile_fp64(const StepArgs& A, const PatchDev&
 }
 
 // ------------------------------------------------------------------------- the kernel
-// STAGE: two buffers, filled by 0 asynchronous 8-byte copies, 1 tensor bulk copies; 2 tensor bulk copies into one (the next tile's copy
-// is requested behind the first barrier, when the tile's state is in registers).  PULL: 1 same-level
-// and boundary ghosts are taken from their source cells; 2 those and the ghosts interpolated from
-// the coarser level, evaluated in the step.
+// STAGE: two buffers, filled by 0 asynchronous 8-byte copies, 1 tensor bulk copies; 2 tensor bulk copies into
+// one (the next tile's copy is requested behind the first barrier, when the tile's state is in registers).
+// PULL: 1 same-level and boundary ghosts are taken from their source cells; 2 those and the ghosts
+// interpolated from the coarser level, evaluated in the step.
 template <int LIM, int TX, int TY, int NT, int STAGE, int PULL>
 __global__ void __launch_bounds__(NT, NT == 128 ? 4 : NT == 256 ? (TY == 16 ? 3 : 2) : NT == 352 ? 2 : NT == 192 ? 3 : 1)
     uniform_step_kernel(const __grid_constant__ StepArgs A)
 {
-    using U = UniGeo<TX, TY, NT>;
+    using U = UniGeo<TX, TY, NT, STAGE>;
     using G = Geo<TX, TY>;
     constexpr bool TWO = STAGE != 2;
     constexpr int NBUF = TWO ? 2 : 1;
@@ -245,7 +248,7 @@ __global__ void __launch_bounds__(NT, NT == 128 ? 4 : NT == 256 ? (TY == 16 ? 3 
     double* qbuf = smem;                              // NBUF x QSTRIDE
     double* work = smem + NBUF * G::QSTRIDE;
     double* frame = work + U::WORK;                   // side buffer of the pulled ghosts: 3 planes of NF
-    unsigned long long* bar = reinterpret_cast<unsigned long long*>(frame + U::side(STAGE, PULL));
+    unsigned long long* bar = reinterpret_cast<unsigned long long*>(frame + U::side(PULL));
     __shared__ PatchDev s_patch[2];                   // the tile's box, by tile parity
     __shared__ fx::Shared s_fx;
     __shared__ int s_flag;
@@ -466,7 +469,7 @@ __global__ void __launch_bounds__(NT, NT == 128 ? 4 : NT == 256 ? (TY == 16 ? 3 
             A, P, s_fx, s_fx.run[fx_set], par, sq, work, A.Z0, T.tx, T.ty, T.x0, T.y0, my_flag, jumps_done, begin,
             strengths_done, limited_done);
         if (!done) {
-            my_flag |= uniform_tile_fp64<LIM, TX, NT>(A, P, sq, G::QPL, work, T.tx, T.ty, T.x0, T.y0);
+            my_flag |= uniform_tile_fp64<LIM, TX, U::FP64_ROWS, NT>(A, P, sq, G::QPL, work, T.tx, T.ty, T.x0, T.y0);
             begin();
             strengths_done();
             if (PULL && STAGE == 0) __syncthreads();
@@ -491,7 +494,7 @@ template <int LIM, int TX, int TY, int NT, int STAGE, int PULL> StepKernel unifo
 {
     StepKernel k;
     k.fn = uniform_step_kernel<LIM, TX, TY, NT, STAGE, PULL>;
-    k.smem = UniGeo<TX, TY, NT>::smem(STAGE, PULL);
+    k.smem = UniGeo<TX, TY, NT, STAGE>::smem(PULL);
     k.nt = NT;
     return k;
 }

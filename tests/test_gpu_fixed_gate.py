@@ -113,3 +113,26 @@ def test_small_states_beside_a_large_jump_keep_their_precision(ratio, order, tra
         else:
             bound = np.array([2.02, 1.02, 1.02] if order == 1 else [5.06, 3.06, 3.06])
         assert np.all(rel <= bound), (rel, bound)
+
+
+@pytest.mark.parametrize("tiling", [(32, 32, 1, 256), (32, 32, 0, 512), (32, 16, 2, 256), (16, 16, 1, 128), (16, 16, 0, 192)])
+def test_a_state_without_jumps_comes_out_as_it_is(tiling):
+    # bit for bit, signs of zeros included, whatever its size
+    for state in ((0.0, 0.0, 0.0), (0.0, -0.0, 0.0), (-0.0, 0.0, -0.0), (5.0e-324, 0.0, 0.0), (1.0e-310, -1.0e-312, 3.0e-320),
+                  (1.0e-290, 0.0, -1.0e-300), (1.0, -0.0, 1.0e-300), (1.0e300, 1.0e290, 0.0)):
+        q = np.broadcast_to(np.array(state)[:, None, None], (3, 52, 70)).copy()
+        got, _ = _step(q, 0.9, 0.02, 2, 2, 4, tiling)
+        assert np.array_equal(got.view(np.int64), q[:, 2:-2, 2:-2].copy().view(np.int64))
+
+
+def test_the_smallest_jumps_are_not_taken_for_none():
+    # subnormal jumps, whose upper words are zero, on zeros: some of it moves on, as the exact step has it within a
+    # unit of the smallest subnormal for each of the FP64 phases' operations (24 for all terms of p)
+    for size in (2.0 ** -1043, 2.0 ** -1060):
+        q = np.zeros((3, 52, 52))
+        q[0, 24:28, 24:28] = size
+        got, nu = _step(q, 0.9, 0.02, 2, 2, 4, (32, 32, 1, 256))
+        want = _want(q, nu, 2, 2)
+        assert np.abs(got - want).max() <= 24 * 2.0 ** -1074
+        assert np.count_nonzero(got[1]) > 8 and np.abs(got[1]).max() > size / 8
+        assert not got[:, :16, :16].any()
