@@ -36,9 +36,9 @@
 //   PD  transverse differences, 3 x 8                                        24
 //   total 324 (the tile's halo adds about a third in the kernel).
 // The kernel issues fewer: reciprocals in three instructions (swe::recip), halvings and doublings in
-// the exponent field, h_p in three a wave, and a subcritical edge's side in 30 (PC), four
+// the exponent field, a1 + a3 = dh, h_p in three a wave, and a subcritical edge's side in 30 (PC), four
 // less where the cell's sums start, un +- c stored per edge (2764 us a step without the stored ones).
-// 2048^2 in patches of 32^2: 3401 us a step before all of these, 2688 now; it is bound by the FP64 pipe
+// 2048^2 in patches of 32^2: 3401 us a step before all of these, 2667 now; it is bound by the FP64 pipe
 // (83 % of its nominal rate, which measures 84-90 % at best).
 #pragma once
 
@@ -96,17 +96,6 @@ __device__ __forceinline__ double recip(double x)
     const double e = fma(-x, r, 1.0);
     const double y = fma(r, fma(e, e, e), r);
     return (__double2hiint(x) & 0x7fffffff) == 0x7ff00000 ? r : y;   // (an infinity: e is NaN; NaNs here are quiet)
-}
-// wave strengths of an edge from its Roe state (s1, s3 = un -+ c, ut, i2c = 1 / (2 c)) and jumps of (h, normal,
-// tangential momentum).  a3 is not formed as dh - a1, an instruction less: where the third wave is all but
-// absent that leaves a1's rounding, three times the error (rms 7e-17 |dh| against 2.4e-17; 2048^2: 2667
-// us a step so, 2688 like this).
-__device__ __forceinline__ void strengths(double s1, double s3, double ut, double i2c, double dh, double dn, double dt,
-                                          double& a1, double& a2, double& a3)
-{
-    a1 = fma(s3, dh, -dn) * i2c;
-    a2 = fma(-ut, dh, dt);
-    a3 = fma(-s1, dh, dn) * i2c;
 }
 // x / 2 and 2 x in the exponent field (integer pipe), for 0 and where x and the result are normal; infinities and
 // NaN stay what they are
@@ -358,17 +347,23 @@ __global__ void __launch_bounds__(NT, 1) swe_step_kernel(const __grid_constant__
                 XE[S::XE + e] = ut;
                 XE[2 * S::XE + e] = c;
                 XE[3 * S::XE + e] = i2c;
-                const double s1 = un - c, s3 = un + c;
-                double a1, a2, a3;
-                swe::strengths(s1, s3, ut, i2c, dh, dn, dtg, a1, a2, a3);
+                // a1 = ((un + c) dh - dn) / 2c, and a1 + a3 = dh: an instruction less than both from the speeds, and
+                // the waves then carry the jump exactly.  An absent third wave keeps a1's rounding so (7e-17 |dh|
+                // rms against 2e-17), but the step's results are closer to extended precision: rms of hu, hv
+                // 4.3e-17 against 5.6e-17 of h over blocks of depths from 0.05 to 1, 4.5e-18 against 4.8e-18
+                // on smooth waves, h as before or better.
+                const double a1 = fma(fma(un, dh, -dn), i2c, swe::half(dh));
                 XE[4 * S::XE + e] = a1;
-                XE[5 * S::XE + e] = a2;
-                XE[6 * S::XE + e] = a3;
+                XE[5 * S::XE + e] = fma(-ut, dh, dtg);
+                XE[6 * S::XE + e] = dh - a1;
                 if (!WALK) {
+                    const double s1 = un - c, s3 = un + c;
                     XE[7 * S::XE + e] = s1;
                     XE[8 * S::XE + e] = s3;
+                    if (a >= 0 && a <= tx) m = umax64(m, umax64(swe::mag(s1), swe::mag(s3)));
+                } else if (a >= 0 && a <= tx) {
+                    m = umax64(m, swe::mag(fabs(un) + c));   // max(|un - c|, |un + c|), c > 0
                 }
-                if (a >= 0 && a <= tx) m = umax64(m, umax64(swe::mag(s1), swe::mag(s3)));
             }
         }
         {   // y-edge b (rows b-1 | b) on columns c in [-1, tx]; normal momentum hv
@@ -388,17 +383,19 @@ __global__ void __launch_bounds__(NT, 1) swe_step_kernel(const __grid_constant__
                 YE[S::YE + e] = ut;
                 YE[2 * S::YE + e] = c;
                 YE[3 * S::YE + e] = i2c;
-                const double s1 = un - c, s3 = un + c;
-                double a1, a2, a3;
-                swe::strengths(s1, s3, ut, i2c, dh, dn, dtg, a1, a2, a3);
+                // a1 = ((un + c) dh - dn) / 2c, and a1 + a3 = dh
+                const double a1 = fma(fma(un, dh, -dn), i2c, swe::half(dh));
                 YE[4 * S::YE + e] = a1;
-                YE[5 * S::YE + e] = a2;
-                YE[6 * S::YE + e] = a3;
+                YE[5 * S::YE + e] = fma(-ut, dh, dtg);
+                YE[6 * S::YE + e] = dh - a1;
                 if (!WALK) {
+                    const double s1 = un - c, s3 = un + c;
                     YE[7 * S::YE + e] = s1;
                     YE[8 * S::YE + e] = s3;
+                    if (bb >= 0 && bb <= ty) m = umax64(m, umax64(swe::mag(s1), swe::mag(s3)));
+                } else if (bb >= 0 && bb <= ty) {
+                    m = umax64(m, swe::mag(fabs(un) + c));   // max(|un - c|, |un + c|), c > 0
                 }
-                if (bb >= 0 && bb <= ty) m = umax64(m, umax64(swe::mag(s1), swe::mag(s3)));
             }
         }
 #pragma unroll
