@@ -131,6 +131,9 @@ int claw_set_level(claw_ctx* ctx, int32_t level, const claw_box* boxes, int32_t 
  * shallow water: 16x16 with 256 threads, 32x16 with 512; claw_set_level installs 16x16.  Once
  * chosen here, a level's tiling stays through later claw_set_level calls (with staging 0 when
  * the new boxes do not allow bulk copies), as does its claw_set_tile_walk choice.
+ * In a uniform medium the step works in units that follow a tile's largest jump: q_new agrees to rounding
+ * between tilings (and between boxes that cut the tiles differently), not bit for bit, and a program
+ * that wants the same bits from run to run sets the tiling itself.
  * Staging 1 is installed when allowed.  A new tile shape rewrites the level's tile lists in
  * place (after synchronising the device): graphs captured before must not be replayed.
  * Errors: CLAW_EINVAL, CLAW_ENOMEM, CLAW_ECUDA. */

@@ -13,7 +13,10 @@ namespace claw {
 constexpr int kAverageThreads = 128;
 
 // chunks a rectangle is split into, for rectangles of up to max_cells coarse cells
-inline int average_chunks(int max_cells) { return std::max(1, std::min(64, (3 * max_cells + kAverageThreads - 1) / kAverageThreads)); }
+inline int average_chunks(int max_cells)
+{
+    return std::max(1, std::min(64, (3 * max_cells + kAverageThreads - 1) / kAverageThreads));
+}
 inline int average_blocks(int nrects, int max_cells) { return nrects <= 0 ? 0 : nrects * average_chunks(max_cells); }
 
 // the r x r children are summed row by row and divided by r^2 (an exact product for r = 2, 4), all of

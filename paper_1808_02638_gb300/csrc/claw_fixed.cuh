@@ -11,17 +11,17 @@
 //
 // Precision: with e such that |du|, |dv|, |dp| / Z < 2^e on every edge of the tile, by their exponents and that
 // of 1 / Z, the unit is 2^(e - 58).  Sums and limiters are exact (van Leer's quotient within 7 units of
-// M, see below), a product errs by at most 0.75 units.  An increment of p / Z, u or v errs by up to 5
+// M, see below), a product errs by at most one unit.  An increment of p / Z, u or v errs by up to 5
 // units, 1.3 rms (emulated, uniformly random states with exact jumps: all limiters, orders and
-// transverse modes); the bound by adding all up is 25.
+// transverse modes); adding up every bound gives some 40.
 //
 // A tile is stepped this way only if at every edge the state next to it or the jump across it, the largest
 // of |p| / Z, |u| and |v|, is at least 2^(e - 4): 5 units are then 2.5 roundings (2^-53) of that state, and
 // the fused multiply-add that forms the result is the one other.  The FP64 phases take five such
 // operations for p and three for u and v.  Emulated, relative to the state, in cells beside a
-// jump at that limit: at most 2.4 and 1.7 roundings (p; u and v), 0.72 and 0.58 rms, where the FP64 phases
+// jump at that limit: at most 2.5 and 1.7 roundings (p; u and v), 0.72 and 0.59 rms, where the FP64 phases
 // have 4.4 and 2.9, 1.2 and 0.94.  The first-order step has two and one operations without transverse
-// terms (2.0 and 1.0 roundings at most; fixed point 1.5 and 1.2 at 2^(e - 4)): it takes fixed point
+// terms (2.0 and 1.0 roundings at most; fixed point 1.8 and 1.2 at 2^(e - 4)): it takes fixed point
 // from 2^(e - 2) on.
 //
 // The precision is that of the state as a vector in wave units.  A component far smaller than the others and
@@ -29,13 +29,13 @@
 // absolute error, 2^-56 of the largest jump, not to its own last bits as in FP64.
 //
 // Every other tile (a front on a zero background, infinities, NaN, extreme exponents, a CFL number above 1 in
-// either direction) takes the FP64 phases, 2.5 times as long; a tile without any jump does not, whatever its
+// either direction) takes the FP64 phases, 2.6 times as long; a tile without any jump does not, whatever its
 // state.  Path and unit depend on the states of the tile alone: how it was staged or who stepped it does
 // not matter, but its shape does.  Two tilings of the same state agree to rounding, not bit for bit.
 //
 // What bounds it: the latency of dependent integer chains at 16 warps an SM; no pipe is at its limit (the ALU
 // is the busiest), and FP64 and memory no longer are.  2048^2 in patches of 32^2 with pulled ghosts, MC
-// limiter: 412 us a step when all of it was FP64, 193 now; 1001 x 604 in ragged patches, van Leer: 146 and
+// limiter: 412 us a step when all of it was FP64, 185 now; 1001 x 604 in ragged patches, van Leer: 146 and
 // 47 (the FP64 reciprocals went).
 #pragma once
 
@@ -45,36 +45,37 @@ namespace claw {
 namespace fx {
 
 // ------------------------------------------------------------------------- numbers
-// a constant c in [0, 1/4]: c = (hi 2^32 + lo) / 2^64, lo signed, 0 <= hi <= 2^30
+// a constant c in [0, 1/4]: c = (hi 2^32 + lo) / 2^64, hi <= 2^30
 struct __align__(16) Coef {
-    int hi, lo;
+    unsigned hi, lo;
     unsigned half;   // 2^31 + lo / 2: half a unit, and the mean of the product that mul drops
 };
 __device__ __forceinline__ Coef coef_bits(long long c)   // c 2^64, at most 2^62
 {
     Coef r;
-    r.lo = (int)(unsigned)c;
-    r.hi = (int)((c - r.lo) >> 32);
-    r.half = 0x80000000u + (unsigned)(r.lo >> 1);
+    r.lo = (unsigned)c;
+    r.hi = (unsigned)(c >> 32);
+    r.half = 0x80000000u + (r.lo >> 1);
     return r;
 }
 
 // Rounding: products and conversions are of magnitudes, to nearest, and take the sign afterwards; quarters
 // round halves to even.  Results are then odd functions of their arguments, so that a mirror-symmetric
-// state stays so bit for bit, and their errors have no preferred sign.  Rounding downwards instead (184
-// against 193 us a step of 2048^2) let the total of p drift by 6e-15 a step on 64^2 cells, linearly; like
-// this it wanders no further than that of the FP64 phases.
+// state stays so bit for bit, and their errors have no preferred sign.  Rounding downwards instead let
+// the total of p drift by 6e-15 a step on 64^2 cells, linearly; like this it wanders no further than that
+// of the FP64 phases.  (2048^2 took the same time so, 1001 x 604 with van Leer 44 us against 47.)
 
-// w c for a magnitude w < 2^63, within 0.75 units: the product of the low words, between -1/2 and 1/2 units,
-// is replaced by its mean.  0 gives 0: where nothing changes, nothing may.
+// w c for a magnitude w < 2^63, within a unit: the product of the low words, below one, is replaced by its mean.
+// 0 gives 0: where nothing changes, nothing may.  (All unsigned: with a signed lo, whose sum of cross products
+// is signed too, 2048^2 took 192 us a step, 185 so.)
 __device__ __forceinline__ long long mul_mag(long long w, Coef c)
 {
-    const int wh = (int)(w >> 32);
-    long long x = (long long)wh * c.lo + (long long)(unsigned long long)c.half;   // cross products, units / 2^32
-    x += (long long)((unsigned long long)(unsigned)w * (unsigned)c.hi);           // below 2^62 each
-    return (long long)wh * c.hi + (int)(x >> 32);
+    const unsigned wh = (unsigned)(w >> 32);
+    unsigned long long x = (unsigned long long)wh * c.lo + c.half;   // cross products, units / 2^32: below 2^63 + 2^62
+    x += (unsigned long long)(unsigned)w * c.hi;
+    return (long long)((unsigned long long)wh * c.hi + (x >> 32));
 }
-// m with its sign changed if s < 0.  (A select: exclusive or and difference took 203 against 193 us a step of
+// m with its sign changed if s < 0.  (A select: exclusive or and difference took 203 against 194 us a step of
 // 2048^2.)
 __device__ __forceinline__ long long signed_by(long long m, int s) { return s < 0 ? -m : m; }
 __device__ __forceinline__ int sign_of(long long v) { return (int)(v >> 32); }
@@ -390,7 +391,7 @@ __device__ __forceinline__ bool step_tile(const StepArgs& A, const PatchDev& P, 
     fine = fine && e >= 500 && e <= 1600 && (mn >> 20) >= ((mp | mu) ? least : 100);
     if (!fine && run.ok && (mp | mu) == 0u) {
         // a tile whose jumps are zero to the last bit comes out as it is, in integers as in FP64, however small its
-        // state.  (Zeros in front of a wave, the whole of 2048^2: 507 us by the FP64 phases, 217 so.)
+        // state.  (Zeros in front of a wave, the whole of 2048^2: 507 us by the FP64 phases, 211 so.)
         bool still = true;
 #pragma unroll
         for (int j = 0; j < R; ++j) {

@@ -288,12 +288,15 @@ cudaError_t launch_average_adjoint(const AvgRect* r, int n, int ratio, double* l
 // ------------------------------------------------------------------------ box-wise kernels
 // blocks of (box, chunk of kBoxRows rows, share of the chunk): a level of few boxes has few chunks, and 17
 // blocks of 128 threads (a box of 256^2) kept 17 SMs busy with some 30 rounds of square roots and divisions.
-// The chunks of such a level are shared by up to `most` blocks each, until there are about eight per SM:
-// medium planes of 256^2 137 us before, 22 us now, their adjoint 432 and 61.
+// The chunks of such a level are shared by up to `most` blocks each, until there are about eight per SM of the
+// part: medium planes of 256^2 137 us before, 22 us now, their adjoint 432 and 61.  `most` leaves a thread, of a
+// chunk of 256 columns, one cell of the medium planes, three elements of a packed copy, and four cells of
+// a speed maximum, whose blocks end in an atomic each.
+constexpr long long kBoxBlocks = 8 * 152;
 static inline dim3 box_rows_grid(int n, int max_rows, int most)
 {
     const int chunks = (max_rows + kBoxRows - 1) / kBoxRows;
-    const long long share = 1216 / ((long long)n * chunks);
+    const long long share = kBoxBlocks / ((long long)n * chunks);
     return dim3((unsigned)n, (unsigned)chunks, (unsigned)std::max(1LL, std::min<long long>(share, most)));
 }
 

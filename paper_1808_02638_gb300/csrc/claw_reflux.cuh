@@ -114,8 +114,9 @@ __device__ __forceinline__ void edge_terms(const Row& row, int lane, const StepA
 }
 
 // ------------------------------------------------------------------ shallow water
-// Roe state and wave strengths of one edge (the step kernel's formulation: per-cell sqrt(h) and
-// momenta over sqrt(h), one reciprocal, one reciprocal square root for c and 1/(2c))
+// Roe state and wave strengths of one edge: the step kernel's to rounding (per-cell sqrt(h) and momenta over
+// sqrt(h), one reciprocal square root for c and 1/(2c); here the reciprocal is a division's and the
+// third strength comes from its own speed)
 struct SEdge {
     double un, ut, c, i2c, a1, a2, a3;
 };

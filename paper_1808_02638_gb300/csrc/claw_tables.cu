@@ -167,7 +167,8 @@ static void deal(std::vector<TileDev>& t, int nsm)
 // The largest number of rows of a level's tiles, at most ty, for the kernels bound by the FP64 pipe: a
 // level of few tiles leaves SMs idle, or gives some two tiles and others one, and lower tiles fill
 // them.  The work of a tile is about its cells with the halo of its edges and a share for its
-// latency; the busiest SM decides.  Measured, full rows and lower ones: cell-wise medium 256^2
+// latency; the busiest SM decides (2.7 rows, 36 cells and the 3 % below, under which no lower tile is
+// taken, are fitted to launches over such levels, in cells of either system).  Measured, full rows and lower ones: cell-wise medium 256^2
 // on 32 x 16 tiles 21.4 and 19.3 us (14 rows: 152 tiles for 152 SMs), 190 x 170 21.1 and 14.8 (8 rows); shallow
 // water 64^2 on 16 x 16 tiles 34.1 and 19 us (6 rows), 24 boxes with 14256 cells 35 and 24.  Past two
 // tiles an SM nothing is gained.  The uniform medium's integer step gains at most 3 % (100^2:
